@@ -183,8 +183,9 @@ namespace {
 constexpr uint32_t WINDOWS_PER_TASK = 16;
 constexpr int SK_NW = 2;  // windows sketched together by a warp
 
-// One warp per window; a warp takes WINDOWS_PER_TASK consecutive windows
-// and walks the sequences they belong to.  EMIT = build pairs, else the
+// One warp per window (sketch sizes above 16, which lane_sketch does not
+// take); a warp takes WINDOWS_PER_TASK consecutive windows and walks the
+// sequences they belong to.  EMIT = build pairs, else the
 // debug sketch export.  Five resident blocks per SM (48 registers).
 template <int R, int KC, bool EMIT>
 __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq, const uint8_t* __restrict__ seq,
@@ -252,16 +253,194 @@ __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq
     if (EMIT && lane == 0 && real) atomicAdd(real_pairs, real);
 }
 
+// The same work with one window per lane (lane_sketch, sketch sizes up to
+// 16): a warp takes 32 consecutive windows at a time, stages the bases they
+// cover as 2-bit codes in shared memory (each base loaded and encoded once,
+// 16 bytes a lane), sketches them together and writes their pairs, which are
+// consecutive in memory, through shared memory with whole-line stores.
+// Windows of consecutive targets are in memory order too; should targets too
+// short for a window lie between them and spread the 32 windows over more
+// bytes than the staging area holds, the windows that fit are taken first.
+// A window that lane_sketch does not settle is sketched by the whole warp.
+// Bound by the integer ALU (half the issue rate): 14.3 Gbp of the large
+// workload take 22.4 ms (127 M windows of 113 k-mers), against 64.5 ms with
+// one warp per window; 25.9, 23.6 and 22.4 ms at 4, 5 and 6 CTAs per SM.
+constexpr uint32_t EMIT_CAP = 48;  // candidates per lane
+__host__ __device__ inline uint32_t emit_stage_words(const SketchParams& p) {
+    return (31 * p.stride + p.w + 30) / 16 + 2;
+}
+__host__ __device__ inline size_t emit_warp_bytes(const SketchParams& p) {
+    const size_t words = emit_stage_words(p);
+    return words * 4 + ((words * 2 + 3) & ~(size_t)3) + ls_cand_words(EMIT_CAP) * 4;
+}
+constexpr int EMIT_WARPS = 4;
+constexpr int EMIT_CTAS = 6;  // resident per SM: 80 registers, 34 KB of shared memory each
+
+template <int R, int KC, bool EMIT>
+__global__ void __launch_bounds__(EMIT_WARPS * 32, EMIT_CTAS)
+    k_sketch_lanes(SketchParams p, uint32_t n_seq, const uint8_t* __restrict__ seq, const uint64_t* __restrict__ offs,
+                   const uint64_t* __restrict__ win_offs, uint64_t n_windows, uint32_t task_windows, uint32_t gw_base,
+                   uint64_t* __restrict__ pairs, uint32_t* __restrict__ sketch, uint32_t* __restrict__ counts,
+                   unsigned long long* real_pairs) {
+    extern __shared__ __align__(16) unsigned char emit_smem[];
+    const uint32_t lane = lane_id();
+    const uint32_t n_words = emit_stage_words(p);
+    uint32_t* code = reinterpret_cast<uint32_t*>(emit_smem + (threadIdx.x >> 5) * emit_warp_bytes(p));
+    uint32_t* cand = code + n_words;  // candidates, then the features
+    uint16_t* inv = reinterpret_cast<uint16_t*>(cand + ls_cand_words(EMIT_CAP));
+    const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t k = KC ? (uint32_t)KC : p.k;
+    unsigned long long real = 0;
+    for (uint64_t w0 = warp * task_windows; w0 < n_windows; w0 += n_warps * task_windows) {
+        const uint64_t w1 = min(w0 + task_windows, n_windows);
+        uint32_t t = 0;  // last target with win_offs[t] <= the round's first window
+        {
+            uint32_t hi = n_seq;
+            while (hi - t > 1) {
+                const uint32_t mid = (t + hi) >> 1;
+                if (win_offs[mid] <= w0) t = mid; else hi = mid;
+            }
+        }
+        for (uint64_t x0 = w0; x0 < w1; x0 += 32) {
+            const uint64_t x = min(x0 + lane, w1 - 1);
+            const bool act = x0 + lane < w1;
+            uint32_t tl = t;
+            if (win_offs[t + 1] <= min(x0 + 31, w1 - 1)) {  // the round leaves target t
+                uint32_t hi = n_seq;
+                while (hi - tl > 1) {
+                    const uint32_t mid = (tl + hi) >> 1;
+                    if (win_offs[mid] <= x) tl = mid; else hi = mid;
+                }
+            }
+            t = __shfl_sync(FULL_MASK, tl, 31);  // a later target or the same for the next round
+            const uint64_t L = offs[tl + 1] - offs[tl];
+            const uint64_t ws = (x - win_offs[tl]) * p.stride;
+            const uint32_t n_k = window_kmers(L, ws, p);
+            const uintptr_t first = reinterpret_cast<uintptr_t>(seq) + offs[tl] + ws;
+            const uintptr_t end = first + n_k + k - 1;
+            uint32_t todo = __ballot_sync(FULL_MASK, act);
+            while (todo) {
+                // the run of windows from the first one left whose bases fit
+                const uint32_t lead = __ffs(todo) - 1;
+                const uintptr_t f0 = __shfl_sync(FULL_MASK, first, lead);
+                const uintptr_t a0 = f0 & ~(uintptr_t)15;
+                const uint32_t fits = __ballot_sync(FULL_MASK, ((todo >> lane) & 1u) && first >= f0 &&
+                                                                   end <= a0 + (uintptr_t)(n_words - 1) * 16);
+                const uint32_t run = fits >> lead;  // bit 0 is set: one window always fits
+                const uint32_t n_now = run == FULL_MASK ? 32u : __ffs(~run) - 1;
+                const bool in = lane - lead < n_now;
+                todo &= ~((n_now == 32 ? FULL_MASK : (1u << n_now) - 1u) << lead);
+                const uint32_t n_ch = (__reduce_max_sync(FULL_MASK, in ? (uint32_t)(end - a0) : 0u) + 15) / 16;
+                // bytes outside the targets of these windows are not read
+                const uintptr_t lo = reinterpret_cast<uintptr_t>(seq) + __shfl_sync(FULL_MASK, offs[tl], lead);
+                const uintptr_t t_end = reinterpret_cast<uintptr_t>(seq) + offs[tl + 1];
+                const uintptr_t hi =
+                    a0 + __reduce_max_sync(FULL_MASK, in ? (uint32_t)min(t_end - a0, (uintptr_t)0x7FFFFFFF) : 0u);
+                __syncwarp();
+                uint32_t bad = 0;
+                if (a0 >= lo && a0 + 16 * (uintptr_t)n_ch <= hi) {
+                    for (uint32_t c = lane; c < n_ch; c += 32) {
+                        uint32_t iv;
+                        code[c] = encode16(__ldg(reinterpret_cast<const uint4*>(a0) + c), iv);
+                        inv[c] = (uint16_t)iv;
+                        bad |= iv;
+                    }
+                } else {
+                    for (uint32_t c = lane; c < n_ch; c += 32) {
+                        uint32_t iv;
+                        code[c] = encode16(load_chunk(a0 + 16 * (uintptr_t)c, lo, hi), iv);
+                        inv[c] = (uint16_t)iv;
+                        bad |= iv;
+                    }
+                }
+                const bool any_inv = __any_sync(FULL_MASK, bad != 0);
+                __syncwarp();
+                uint32_t v[16], cnt;
+                const bool ok = lane_sketch<KC, EMIT_CAP>(code, inv, n_ch, any_inv, in ? (uint32_t)(first - a0) : 0u,
+                                                in ? n_k : 0u, p, cand, v, cnt);
+                uint32_t again = __ballot_sync(FULL_MASK, in && !ok);
+                __syncwarp();  // the candidates are read: the buffer now takes the features
+                uint32_t* feat = cand;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) feat[i * LS_FEAT_STRIDE + lane] = v[i];
+                while (again) {  // exact selection by the whole warp
+                    const uint32_t l = __ffs(again) - 1;
+                    again &= again - 1;
+                    const uint32_t ta = __shfl_sync(FULL_MASK, tl, l);
+                    const uint8_t* const sq[1] = {seq + offs[ta]};
+                    const uint64_t Ls[1] = {__shfl_sync(FULL_MASK, L, l)}, wss[1] = {__shfl_sync(FULL_MASK, ws, l)};
+                    const bool on[1] = {true};
+                    uint32_t f[1], c1[1];
+                    __syncwarp();
+                    warp_sketch_multi<R, 1, KC>(sq, Ls, wss, on, p, feat + 16 * LS_FEAT_STRIDE, f, c1);
+                    if (lane < c1[0]) feat[lane * LS_FEAT_STRIDE + l] = f[0];
+                    if (lane == l) cnt = c1[0];
+                }
+                __syncwarp();
+                if (!in) cnt = 0;
+                real += cnt;
+                if (!EMIT && in) counts[x] = cnt;
+                // entry e of the round's n_now * s outputs: feature e % s of window e / s
+                const uint64_t out0 = (x0 + lead) * p.s;
+                for (uint32_t e0 = 0; e0 < n_now * p.s; e0 += 32) {
+                    const uint32_t e = e0 + lane;
+                    const uint32_t wl = p.s == 16 ? e >> 4 : e / p.s;
+                    const uint32_t i = e - wl * p.s;
+                    const uint32_t src = (lead + wl) & 31u;
+                    const uint32_t c = __shfl_sync(FULL_MASK, cnt, src);
+                    if (wl < n_now) {
+                        const uint32_t fv = feat[i * LS_FEAT_STRIDE + src];
+                        if (EMIT)
+                            pairs[out0 + e] = i < c ? (((uint64_t)hash_h2(fv) << 32) |
+                                                       (uint32_t)(gw_base + x0 + lead + wl))
+                                                    : SENTINEL_PAIR;
+                        else
+                            sketch[out0 + e] = i < c ? fv : 0u;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+    if (EMIT) {
+        for (int o = 16; o >= 1; o >>= 1) real += __shfl_xor_sync(FULL_MASK, real, o);
+        if (lane == 0 && real) atomicAdd(real_pairs, real);
+    }
+}
+
 template <bool EMIT>
 cudaError_t launch_sketch(const SketchParams& p, uint32_t n_seq, const uint8_t* seq, const uint64_t* offs,
                           const uint64_t* win_offs, uint64_t n_windows, uint32_t gw_base, uint64_t* pairs,
                           uint32_t* sketch, uint32_t* counts, unsigned long long* real, cudaStream_t s) {
     if (n_windows == 0) return cudaSuccess;
+    const int r = sketch_r_for(p.w);
+    const char* name = EMIT ? "sketch_emit" : "sketch";
+    if (p.s <= LS_MAX_S) {
+        using Kernel = void (*)(SketchParams, uint32_t, const uint8_t*, const uint64_t*, const uint64_t*, uint64_t,
+                                uint32_t, uint32_t, uint64_t*, uint32_t*, uint32_t*, unsigned long long*);
+        const bool k16 = p.k == 16;
+        const Kernel kern = r == 4   ? (k16 ? k_sketch_lanes<4, 16, EMIT> : k_sketch_lanes<4, 0, EMIT>)
+                            : r == 8 ? (k16 ? k_sketch_lanes<8, 16, EMIT> : k_sketch_lanes<8, 0, EMIT>)
+                                     : (k16 ? k_sketch_lanes<16, 16, EMIT> : k_sketch_lanes<16, 0, EMIT>);
+        const size_t smem = EMIT_WARPS * emit_warp_bytes(p);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        // rounds of 32 windows per task: 16 where there are windows enough
+        // for every resident warp, fewer in small calls
+        const uint64_t warps = (uint64_t)NUM_SMS_HINT * 5 * EMIT_WARPS;
+        const uint64_t rounds = (n_windows + 32 * warps - 1) / (32 * warps);
+        const uint32_t task_windows = 32u * (uint32_t)(rounds < 16 ? rounds : 16);
+        const uint64_t tasks = (n_windows + task_windows - 1) / task_windows;
+        const uint32_t g = grid_for((tasks + EMIT_WARPS - 1) / EMIT_WARPS, 20);
+        MC_LAUNCH(name, s,
+                  kern<<<g, EMIT_WARPS * 32, smem, s>>>(p, n_seq, seq, offs, win_offs, n_windows, task_windows,
+                                                        gw_base, pairs, sketch, counts, real));
+        return cudaGetLastError();
+    }
     uint64_t tasks = (n_windows + WINDOWS_PER_TASK - 1) / WINDOWS_PER_TASK;
     uint64_t blocks = (tasks + NWARP - 1) / NWARP;
     uint32_t g = grid_for(blocks, 16);
-    const int r = sketch_r_for(p.w);
-    const char* name = EMIT ? "sketch_emit" : "sketch";
 #define MC_SK(RR, KK) \
     MC_LAUNCH(name, s, k_sketch<RR, KK, EMIT><<<g, BT, 0, s>>>(p, n_seq, seq, offs, win_offs, n_windows, gw_base, pairs, sketch, counts, real))
     if (r == 4) {

@@ -31,14 +31,15 @@ struct SketchParams {
 // ---------------------------------------------------------------- hashing
 // h1: the lowbias32 mixer (C. Wellons, hash-prospector), a bijection on
 // 32-bit words, applied to the canonical k-mer code (Section 4.1).
-__host__ __device__ __forceinline__ uint32_t hash_h1(uint32_t x) {
+__host__ __device__ __forceinline__ uint32_t hash_h1_head(uint32_t x) {
     x ^= x >> 16;
     x *= 0x7feb352dU;
     x ^= x >> 15;
     x *= 0x846ca68bU;
-    x ^= x >> 16;
     return x;
 }
+__host__ __device__ __forceinline__ uint32_t hash_h1_tail(uint32_t x) { return x ^ (x >> 16); }
+__host__ __device__ __forceinline__ uint32_t hash_h1(uint32_t x) { return hash_h1_tail(hash_h1_head(x)); }
 
 // h2: MurmurHash3's 32-bit finalizer, a second bijection used only to place
 // features in the table (Section 4.1: "to counteract the biased distribution

@@ -276,6 +276,230 @@ __device__ __forceinline__ void warp_sketch_multi(const uint8_t* const (&seq)[NW
 }
 
 
+// ------------------------------------------------------ lane-wide sketches
+// The same sketch with one window per lane: a warp sketches 32 windows at
+// once, each lane walking its own window over bases staged in shared memory
+// as 2-bit codes.  What it saves over one warp per window: a k-mer is one
+// funnel shift of two 32-bit words (16 bases) and its reverse complement
+// another (no shuffles, no 64-bit arithmetic), and the selection sorts in
+// registers without cross-lane steps, so that a window costs about 130 warp
+// instructions instead of about 500.  What it needs: 32 windows to fill the
+// warp, and s <= 16.
+
+constexpr uint32_t LS_MAX_S = 16;      // largest sketch size of the lane path
+// words of the candidate buffer for at most cap candidates per lane (eight
+// more rows: the count is checked every 8 k-mers)
+__host__ __device__ constexpr uint32_t ls_cand_words(uint32_t cap) { return (cap + 8) * 32; }
+constexpr uint32_t LS_FEAT_STRIDE = 33;  // feat[i * 33 + lane]: rows and columns without bank conflicts
+constexpr uint32_t LS_MARGIN = 12;     // the cutoff aims at s + 12 candidates
+
+// 16 bases (byte 0 of x = the first) as a 32-bit word of 2-bit codes, first
+// base in the top digit; inv = one bit per invalid base, first base in bit
+// 15.  c is the code of every byte; the letter of a code comes from a byte
+// permute, so a byte is a base iff it equals its own code's letter with bit
+// 5 set.  The invalid bits are only formed when there are some.
+__device__ __forceinline__ uint32_t encode16(const uint4& x, uint32_t& inv) {
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+    uint32_t code = 0, d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t c = ((w[i] >> 1) ^ (w[i] >> 2)) & 0x03030303u;
+        code = (code << 8) | ((c * 0x40100401u) >> 24);
+        const uint32_t n = __byte_perm(c | (c >> 4), 0, 0x4420);  // the four codes as nibbles
+        d[i] = (w[i] | 0x20202020u) ^ __byte_perm(0x74676361u, 0, n);  // 'a' 'c' 'g' 't'
+    }
+    inv = 0;
+    if (d[0] | d[1] | d[2] | d[3]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t z = ((d[i] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | d[i];  // bit 7 of each nonzero byte
+            inv = (inv << 4) | (((((z >> 7) & 0x01010101u) * 0x08040201u) >> 24) & 0xFu);
+        }
+    }
+    return code;
+}
+
+// Reverse complement of 16 bases.
+__device__ __forceinline__ uint32_t revcomp16(uint32_t a) {
+    const uint32_t r = __brev(a);
+    return ~(((r >> 1) & 0x55555555u) | ((r & 0x55555555u) << 1));
+}
+
+// The 16-byte aligned chunk at address c, with bytes outside [lo, hi) left
+// unread (0, an invalid base).
+__device__ __forceinline__ uint4 load_chunk(uintptr_t c, uintptr_t lo, uintptr_t hi) {
+    if (c >= lo && c + 16 <= hi) return __ldg(reinterpret_cast<const uint4*>(c));
+    uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+        if (c + i >= lo && c + i < hi)
+            w[i >> 2] |= (uint32_t)__ldg(reinterpret_cast<const uint8_t*>(c + i)) << (8 * (i & 3));
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Batcher's odd-even merge sort of 16 registers (63 comparators).
+__device__ __forceinline__ void sort16(uint32_t (&v)[16]) {
+#pragma unroll
+    for (int p = 1; p < 16; p <<= 1) {
+#pragma unroll
+        for (int k = p; k >= 1; k >>= 1) {
+#pragma unroll
+            for (int j = k % p; j + k < 16; j += 2 * k) {
+#pragma unroll
+                for (int i = 0; i < k; ++i) {
+                    if (i + j + k < 16 && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+                        const uint32_t a = v[i + j], b = v[i + j + k];
+                        v[i + j] = min(a, b);
+                        v[i + j + k] = max(a, b);
+                    }
+                }
+            }
+        }
+    }
+}
+
+// v = the 16 smallest of the sorted v and u, sorted.
+__device__ __forceinline__ void keep_smallest16(uint32_t (&v)[16], const uint32_t (&u)[16]) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = min(v[i], u[15 - i]);  // bitonic
+#pragma unroll
+    for (int j = 8; j > 0; j >>= 1) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if ((i & j) == 0) {
+                const uint32_t a = v[i], b = v[i | j];
+                v[i] = min(a, b);
+                v[i | j] = max(a, b);
+            }
+        }
+    }
+}
+
+// Keeps y (h1 before its last step) as a candidate if it is at most tau:
+// stored at shared address at, which moves on by one row.
+__device__ __forceinline__ void lane_candidate(uint32_t y, uint32_t tau, uint32_t& at) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.le.u32 p, %1, %2;\n\t"
+        "@p st.shared.u32 [%0], %1;\n\t"
+        "@p add.u32 %0, %0, 128;\n\t}"
+        : "+r"(at)
+        : "r"(y), "r"(tau)
+        : "memory");
+}
+
+// Sketches one window per lane (all lanes of the warp call together).
+//  code, inv : the staged bases (encode16), n_words entries each;
+//  any_inv   : warp-uniform, false if every staged base is valid;
+//  pos, n_k  : this lane's window: staged index of its first base and its
+//              number of k-mers (0 = no window);
+//  cand      : ls_cand_words(CAP) words of the warp's shared memory, for at
+//              most CAP candidates per lane.
+// Returns true if v[0 .. cnt) are the window's features, ascending; false if
+// this lane's window has to be sketched by the exact warp-wide selection:
+// fewer than s candidates below the cutoff, more than CAP, or a repeated
+// value among the s smallest (of random sequence 0.3% of the windows with
+// CAP = 48, 0.7% with CAP = 40).
+// Every word index is clamped to the staged words, so that a lane whose
+// window is shorter than its neighbours' stays inside them.
+template <int KC, uint32_t CAP>
+__device__ __forceinline__ bool lane_sketch(const uint32_t* code, const uint16_t* inv, uint32_t n_words, bool any_inv,
+                                            uint32_t pos, uint32_t n_k, const SketchParams& p, uint32_t* cand,
+                                            uint32_t (&v)[16], uint32_t& cnt) {
+    const uint32_t lane = lane_id();
+    const uint32_t k = KC ? (uint32_t)KC : p.k;
+    const uint32_t aim = p.s + LS_MARGIN;
+    // Any cutoff is correct; a fast reciprocal is plenty for aiming.  Its low
+    // 16 bits are ones: h1's last step y ^= y >> 16 keeps the top 16 bits, so
+    // h1 <= tau iff y <= tau, and only the candidates take that step.
+    const uint32_t tau =
+        n_k <= aim ? 0xFFFFFFFFu : __float2uint_rz(__fdividef((float)aim, (float)n_k) * 4294967296.0f) | 0xFFFFu;
+    const uint32_t n_max = __reduce_max_sync(FULL_MASK, n_k);
+    const uint32_t last = n_words - 1;
+    const uint32_t boff = pos & 15u, sh = 2 * boff;
+    uint32_t wi = pos >> 4;
+    uint32_t w1 = code[min(wi + 1, last)];
+    uint32_t a0 = __funnelshift_l(w1, code[min(wi, last)], sh);
+    uint32_t r0 = revcomp16(a0);
+    // Candidates go to row C of the lane's column: a predicated store and
+    // add each (a branch per k-mer costs more than the k-mer).
+    const uint32_t col = (uint32_t)__cvta_generic_to_shared(cand + lane);
+    const uint32_t col_cap = col + CAP * 128;
+    uint32_t at = col;
+    bool over = false;
+    __syncwarp();  // the candidate buffer may still be read by its previous use
+    for (uint32_t base = 0; base < n_max; base += 16, ++wi) {
+        const uint32_t w2 = code[min(wi + 2, last)];
+        const uint32_t a1 = __funnelshift_l(w2, w1, sh);
+        const uint32_t r1 = revcomp16(a1);
+        // bit 15 - r: k-mer base + r exists and holds no invalid base
+        const uint32_t rem = n_k > base ? n_k - base : 0u;
+        uint32_t ok = rem >= 16 ? 0xFFFFu : (0xFFFF0000u >> rem) & 0xFFFFu;
+        if (any_inv) {
+            const uint32_t hi = ((uint32_t)inv[min(wi, last)] << 16) | inv[min(wi + 1, last)];
+            uint32_t z = __funnelshift_l((uint32_t)inv[min(wi + 2, last)] << 16, hi, boff);
+            uint32_t c = 1;
+            for (; 2 * c <= k; c *= 2) z |= z << c;
+            z |= z << (k - c);
+            ok &= ~(z >> 16);
+        }
+        if (__all_sync(FULL_MASK, ok == 0xFFFFu)) {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                uint32_t f = __funnelshift_l(a1, a0, 2 * r);
+                uint32_t g = __funnelshift_r(r0, r1, 2 * r);
+                if (KC == 0) {
+                    f >>= 32 - 2 * k;
+                    g &= 0xFFFFFFFFu >> (32 - 2 * k);
+                }
+                lane_candidate(hash_h1_head(min(f, g)), tau, at);
+                if ((r & 7) == 7 && at > col_cap) {
+                    over = true;
+                    at = col;
+                }
+            }
+        } else {  // ends of sequences and windows, invalid bases
+            const uint32_t r_max = min(n_max - base, 16u);
+#pragma unroll 1
+            for (uint32_t r = 0; r < r_max; ++r) {
+                uint32_t f = __funnelshift_l(a1, a0, 2 * r);
+                uint32_t g = __funnelshift_r(r0, r1, 2 * r);
+                if (KC == 0) {
+                    f >>= 32 - 2 * k;
+                    g &= 0xFFFFFFFFu >> (32 - 2 * k);
+                }
+                const uint32_t y = hash_h1_head(min(f, g));
+                if ((ok >> (15 - r)) & 1u) lane_candidate(y, tau, at);
+                if (at > col_cap) {
+                    over = true;
+                    at = col;
+                }
+            }
+        }
+        a0 = a1;
+        r0 = r1;
+        w1 = w2;
+    }
+    const uint32_t C = (at - col) >> 7;
+    const uint32_t c_max = __reduce_max_sync(FULL_MASK, C);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0xFFFFFFFFu;
+#pragma unroll 1
+    for (uint32_t b = 0; b < c_max; b += 16) {
+        uint32_t u[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) u[i] = b + i < C ? hash_h1_tail(cand[(b + i) * 32 + lane]) : 0xFFFFFFFFu;
+        sort16(u);
+        keep_smallest16(v, u);
+    }
+    cnt = min(C, p.s);
+    bool dup = false;
+#pragma unroll
+    for (int i = 0; i < 15; ++i) dup |= (uint32_t)(i + 1) < cnt && v[i] == v[i + 1];
+    return !over && !dup && (C >= p.s || tau == 0xFFFFFFFFu);
+}
+
 // R for a window length: the warp covers 32*R >= w bases.
 __host__ __device__ inline int sketch_r_for(uint32_t w) { return w <= 128 ? 4 : (w <= 256 ? 8 : 16); }
 
