@@ -297,11 +297,11 @@ typedef struct mc_batch {
  *  score_mode  : how a query's gathered locations are counted and scored
  *                (the paper's segmented sort, Section 5.5, and window
  *                scoring, Section 5.6): 1 = sort path (default): one warp
- *                gathers the query's locations into registers and sorts
- *                them; 2 = hash path: per-warp hash histogram in shared
- *                memory.  The sort path needs 32-bit locations (mc_db_stats
- *                loc_bytes == 4) and histogram keys of that width
- *                (wide_keys 0); otherwise the hash path is used.
+ *                gathers the query's locations, drops those that cannot
+ *                matter and sorts the rest; 2 = hash path: per-warp hash
+ *                histogram in shared memory.  The sort path takes the
+ *                locations as they are stored (32 or 64 bits); with
+ *                wide_keys 1 on 32-bit locations the hash path is used.
  *  sort_max    : sort path: largest number of gathered locations a query
  *                may have to be sorted, 256, 512, 1024 (default) or 2048; each
  *                size class up to it has its own kernel; larger queries go
@@ -362,7 +362,7 @@ void mc_plan_free(mc_plan* plan);
 
 /* Autotuner: times every lookup setting (probe_batch x lookup_warps) and
  * every score setting (the hash path's hist_slots x gather_batch x
- * score_warps, and, for databases with 32-bit locations, the sort path's
+ * score_warps, and the sort path's
  * sort_max, each with the medium and large paths it leaves) on the given
  * sample batches (at most 2^20 queries
  * in total), `reps` times each, and writes the fastest setting to *best.

@@ -836,6 +836,359 @@ __global__ void __launch_bounds__(LK_WARPS * 32, 4) k_classify_lookup(ClassifyDb
     cp_async_wait_all();
 }
 
+// Main path, part 1 with one window per lane (lane_sketch, sketch sizes up
+// to 16).  A warp takes 2^batch_shift <= 32 consecutive queries, one lane
+// each for their metadata, and works through them in groups that fill its
+// 32 lanes with windows: as many queries as LKL_CHUNKS 16-base chunks and
+// LKL_ITEMS windows hold (16 pairs of 150).  For a group it
+//   - stages the bases as 2-bit codes, a chunk per lane and step;
+//   - lists the windows, whole ones first, so that the lanes of a round
+//     walk windows of like length (a read of 150 has one of 113 k-mers and
+//     one of 22);
+//   - per round of 32 windows sketches them and probes the feature table,
+//     each lane for its own window's features, LB probes in flight.
+// The order of a query's bucket list is of no consequence.
+// Bound by the random reads of the table: 2 M pairs of 150 against the large
+// database (128 M probes of 8.6 GB) take 4.59 ms, 28 G probes/s, against 5.89
+// with one window per warp, which was bound by the sketching; without the
+// probes this kernel takes 1.22 ms.  Entries written one by one instead of
+// through shared memory: 4.87 ms; four or eight probes in flight instead of
+// two: 4.9 and 5.5 ms.
+constexpr uint32_t LKL_CHUNKS = 336;
+constexpr uint32_t LKL_ITEMS = 64;
+constexpr uint32_t LKL_CAP = 40;  // candidates per lane
+constexpr uint32_t LKL_WORDS = (LKL_CHUNKS + 31) / 32 + 1;  // bitmap of chunk starts
+
+struct LookupLanesMem {
+    uint32_t code[LKL_CHUNKS];
+    union {
+        uint32_t cand[ls_cand_words(LKL_CAP)];
+        struct {
+            uint32_t hash[16 * 32];  // [i * 32 + lane]: h2 of a round's features
+            uint32_t exact[32];      // scratch of the exact selection
+            uint16_t more[16 * 32];  // probes to go on with
+            uint64_t found[8 * 32];  // [i * 32 + lane]: buckets found with eight features
+            uint32_t out_start[8];   // bitmap of the lanes' first entries in the output of those
+            uint8_t out_lane[32];    // the lanes that have some, in order
+        };
+        struct {
+            uint64_t base[32];  // chunk c of the group is at base[its query's rank] + 16 c
+            uint32_t starts[LKL_WORDS];
+        } stage;
+    };
+    uint32_t item[LKL_ITEMS];  // staged position | k-mers << 13 | query lane << 23
+    uint32_t q_list[32];       // per query lane: found buckets | features << 16
+    uint32_t q_locs[32];       // locations
+    uint32_t q_sect[32];       // 32-byte sectors
+    uint16_t inv[LKL_CHUNKS];
+};
+static_assert(LKL_CHUNKS * 16 <= 1u << 13, "staged positions take 13 bits");
+
+template <int R, int KC, int LB>
+__global__ void __launch_bounds__(LK_WARPS * 32, 3)
+    k_lookup_lanes(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t chunk, uint32_t list_cap,
+                   uint64_t* __restrict__ glist, uint4* __restrict__ meta, uint32_t* __restrict__ ovf_list,
+                   uint32_t* __restrict__ ovf_n, uint32_t batch_shift) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    LookupLanesMem& M = reinterpret_cast<LookupLanesMem*>(smem)[threadIdx.x >> 5];
+    const uint32_t lane = lane_id();
+    const uint32_t lt = lanemask_lt();
+    const uint32_t le = lt | (1u << lane);
+    const SketchParams& p = db.sp;
+    const uint32_t k = KC ? (uint32_t)KC : p.k;
+    const uint32_t total = total_queries(Q);
+    if (q0 >= total) return;
+    const uint32_t nq = min(chunk, total - q0);
+    const uint64_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nwarp = (gridDim.x * blockDim.x) >> 5;
+    const TableProbe tp(db.fmt);
+    const uint32_t lsz = db.jbits ? 4u : 8u;  // bytes per stored location
+
+    for (uint64_t i0 = gw << batch_shift; i0 < nq; i0 += nwarp << batch_shift) {
+        // one lane per query: size, status, sliding window
+        const uint64_t i = i0 + lane;
+        const bool mine = (lane >> batch_shift) == 0 && i < nq;
+        const uint32_t q = q0 + (uint32_t)i;
+        QueryIn in{};
+        int status = Q_DONE;
+        uint32_t n_win = 0, n_whole = 0, span = 0;
+        uint64_t start = 0;
+        if (mine) {
+            in = query_in(Q, q);
+            if (in.m1 < in.m0 || in.m1 - in.m0 > MAX_MATES) {
+                status = Q_TOO_LARGE;
+            } else {
+                start = in.offs[in.m0];
+                uint64_t o = start, sum = 0, wins = 0;
+                for (uint32_t m = in.m0; m < in.m1; ++m) {
+                    const uint64_t o2 = in.offs[m + 1];
+                    const uint64_t L = o2 > o ? o2 - o : 0;
+                    const uint32_t l = (uint32_t)min(L, (uint64_t)0x7FFFFFFF);  // more is too large anyway
+                    sum += L;
+                    wins += l < k ? 0u : (l - k + p.stride) / p.stride;
+                    n_whole += l < p.w ? 0u : (l - p.w) / p.stride + 1;
+                    o = o2;
+                }
+                if (wins > MC_MAX_QUERY_WINDOWS) status = Q_TOO_LARGE;
+                else if (wins > WIN_A || sum > BUF_A) status = Q_ESCALATE;
+                n_win = (uint32_t)wins;
+                span = (uint32_t)min(sum, (uint64_t)0xFFFFFFFF);
+            }
+            if (status != Q_DONE) {
+                meta[i] = make_uint4(ESCALATED, 0, 0, 0);
+                if (status == Q_ESCALATE) ovf_list[atomicAdd(ovf_n, 1u)] = q;
+                else atomicMax(Q.status, DEV_ERR_CAPACITY);
+            }
+        }
+        for (uint32_t big = __ballot_sync(FULL_MASK, status == Q_TOO_LARGE); big; big &= big - 1)
+            write_unclassified(Q, q0 + (uint32_t)i0 + __ffs(big) - 1);
+        const uintptr_t first = reinterpret_cast<uintptr_t>(in.seq + start);
+        const uint32_t shift = (uint32_t)(first & 15u);
+        const bool active = mine && status == Q_DONE;
+        const uint32_t n_ch = active && n_win ? (shift + span + 15) / 16 : 0u;
+        const uint32_t n_it = active ? n_win : 0u;
+        if (!active) n_whole = 0;
+        M.q_list[lane] = M.q_locs[lane] = M.q_sect[lane] = 0;
+
+        uint32_t todo = __ballot_sync(FULL_MASK, n_it > 0);
+        while (todo) {
+            // the group: queries from the first one left that fit together
+            const bool left = (todo >> lane) & 1u;
+            uint32_t s1 = left ? n_ch | (n_it << 16) : 0u;  // <= 32 * 66 chunks, 32 * 8 windows
+            uint32_t inc = s1;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t x = __shfl_up_sync(FULL_MASK, inc, d);
+                if ((int)lane >= d) inc += x;
+            }
+            const bool in_g = left && (inc & 0xFFFFu) <= LKL_CHUNKS && (inc >> 16) <= LKL_ITEMS;
+            const uint32_t group = __ballot_sync(FULL_MASK, in_g);
+            todo &= ~group;
+            const uint32_t c0 = (inc - s1) & 0xFFFFu;  // first chunk (the group's lanes precede the others left)
+            uint32_t wh = in_g ? n_whole : 0u;
+            uint32_t wh_inc = wh;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t x = __shfl_up_sync(FULL_MASK, wh_inc, d);
+                if ((int)lane >= d) wh_inc += x;
+            }
+            const uint32_t all_whole = __shfl_sync(FULL_MASK, wh_inc, 31);
+            const uint32_t g_last = 31 - __clz(group);
+            const uint32_t n_chunks = __shfl_sync(FULL_MASK, inc, g_last) & 0xFFFFu;
+            const uint32_t n_items = __shfl_sync(FULL_MASK, inc, g_last) >> 16;
+            const uint32_t rank = __popc(group & lt);
+
+            __syncwarp();
+            if (lane < LKL_WORDS) M.stage.starts[lane] = 0;
+            __syncwarp();
+            if (in_g) {
+                M.stage.base[rank] = (uint64_t)(first - shift) - 16 * (uint64_t)c0;
+                atomicOr(&M.stage.starts[c0 >> 5], 1u << (c0 & 31u));
+                // its windows, whole ones first
+                uint32_t whole_at = wh_inc - wh;
+                uint32_t part_at = all_whole + ((inc - s1) >> 16) - (wh_inc - wh);
+                uint32_t pos = c0 * 16 + shift;
+                uint64_t o = start;
+                for (uint32_t m = in.m0; m < in.m1; ++m) {
+                    const uint64_t o2 = in.offs[m + 1];
+                    const uint32_t L = o2 > o ? (uint32_t)(o2 - o) : 0u;  // <= BUF_A
+                    for (uint32_t ws = 0; ws + k <= L; ws += p.stride) {
+                        const uint32_t n_k = min(p.w, L - ws) - k + 1;
+                        const uint32_t at = L - ws >= p.w ? whole_at++ : part_at++;
+                        M.item[at] = (pos + ws) | (n_k << 13) | (lane << 23);
+                    }
+                    pos += L;
+                    o = o2;
+                }
+            }
+            __syncwarp();
+            uint32_t bad = 0, ranks = 0;
+#pragma unroll 1
+            for (uint32_t r = 0; r * 32 < n_chunks; r += 4) {
+                uint4 x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t w = M.stage.starts[min(r + u, LKL_WORDS - 1)];
+                    const uint32_t c = (r + u) * 32 + lane;
+                    if (c < n_chunks)
+                        x[u] = __ldg(reinterpret_cast<const uint4*>(M.stage.base[ranks + __popc(w & le) - 1] +
+                                                                    16 * (uint64_t)c));
+                    ranks += __popc(w);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t c = (r + u) * 32 + lane;
+                    if (c < n_chunks) {
+                        uint32_t iv;
+                        M.code[c] = encode16(x[u], iv);
+                        M.inv[c] = (uint16_t)iv;
+                        bad |= iv;
+                    }
+                }
+            }
+            const bool any_inv = __any_sync(FULL_MASK, bad != 0);
+            __syncwarp();
+
+            for (uint32_t r0 = 0; r0 < n_items; r0 += 32) {
+                const uint32_t it = r0 + lane < n_items ? M.item[r0 + lane] : 0u;
+                const uint32_t pos = it & 0x1FFFu, n_k = (it >> 13) & 0x3FFu, owner = it >> 23;
+                uint32_t v[16], cnt;
+                const bool ok = lane_sketch<KC, LKL_CAP>(M.code, M.inv, n_chunks, any_inv, pos, n_k, p, M.cand, v, cnt);
+                uint32_t again = __ballot_sync(FULL_MASK, !ok);
+                __syncwarp();
+                // (the candidate buffer now takes the features' hashes)
+#pragma unroll
+                for (int x = 0; x < 16; ++x) M.hash[x * 32 + lane] = hash_h2(v[x]);
+                while (again) {  // exact selection by the whole warp
+                    const uint32_t l = __ffs(again) - 1;
+                    again &= again - 1;
+                    const uint32_t lpos = __shfl_sync(FULL_MASK, pos, l), lnk = __shfl_sync(FULL_MASK, n_k, l);
+                    // address of staged position 0 of the lane's query
+                    const uint64_t q_first = (uint64_t)(first - shift) - 16 * (uint64_t)c0;
+                    const uint64_t a = __shfl_sync(FULL_MASK, q_first, __shfl_sync(FULL_MASK, owner, l)) + lpos;
+                    const uint8_t* const sq[1] = {reinterpret_cast<const uint8_t*>(a)};
+                    const uint64_t Ls[1] = {lnk + k - 1}, wss[1] = {0};
+                    const bool on[1] = {true};
+                    uint32_t f[1], c1[1];
+                    warp_sketch_multi<R, 1, KC>(sq, Ls, wss, on, p, M.exact, f, c1);
+                    if (lane < c1[0]) M.hash[lane * 32 + l] = hash_h2(f[0]);
+                    if (lane == l) cnt = c1[0];
+                    __syncwarp();
+                }
+                // Feature table probes: the aligned 16-byte pair of words
+                // holding the home slot; the ordered probe stops at an empty
+                // slot or a key >= h.  The probes that go on beyond their
+                // pair (one in eight) are queued and shared out over the
+                // lanes afterwards, so that a step waits for one load and
+                // not for the longest probe of 32.
+                uint32_t n_more = 0;
+                const auto sectors = [&](uint64_t b) {
+                    const uint64_t lo = (b >> 16) * lsz, hi = lo + (b & 0xFFFFu) * lsz - 1;
+                    return (uint32_t)((hi >> 5) - (lo >> 5) + 1);
+                };
+                const auto queue = [&](bool on, uint32_t entry) {
+                    const uint32_t b = __ballot_sync(FULL_MASK, on);
+                    if (on) M.more[n_more + __popc(b & lt)] = (uint16_t)entry;
+                    n_more += __popc(b);
+                };
+                if (cnt) atomicAdd(&M.q_list[owner], cnt << 16);
+                const uint32_t most = __reduce_max_sync(FULL_MASK, cnt);
+                uint32_t locs = 0, sect = 0;
+#pragma unroll 1
+                for (uint32_t h0 = 0; h0 < most; h0 += 8) {
+                    uint32_t n_f = 0;
+#pragma unroll 1
+                    for (uint32_t b0 = h0; b0 < h0 + 8; b0 += LB) {
+                        ulonglong2 pr[LB];
+#pragma unroll
+                        for (int b = 0; b < LB; ++b) {
+                            const uint32_t home = tp.home(M.hash[(b0 + b) * 32 + lane]);
+                            pr[b] = b0 + b < cnt ? __ldcg(reinterpret_cast<const ulonglong2*>(db.table) + (home >> 1))
+                                                 : make_ulonglong2(0, 0);
+                        }
+#pragma unroll
+                        for (int b = 0; b < LB; ++b) {
+                            const uint32_t h = M.hash[(b0 + b) * 32 + lane];
+                            const uint32_t odd = tp.home(h) & 1u;
+                            uint64_t e = pr[b].x;
+                            uint32_t what = odd ? 2u : tp.step(e, 0, h);
+                            if (what == 2) {
+                                e = pr[b].y;
+                                what = tp.step(e, 1 - odd, h);
+                            }
+                            if (what == 1) {
+                                const uint64_t bk = tp.bucket(e);
+                                M.found[n_f * 32 + lane] = bk;
+                                ++n_f;
+                                locs += (uint32_t)bk & 0xFFFFu;
+                                if (Q.counters) sect += sectors(bk);
+                            }
+                            queue(what == 2, lane | ((b0 + b) << 5));
+                        }
+                    }
+                    // the lanes' entries take the next places of their
+                    // queries' lists; consecutive lanes write consecutive
+                    // entries
+                    uint32_t inc = n_f;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const uint32_t x = __shfl_up_sync(FULL_MASK, inc, d);
+                        if ((int)lane >= d) inc += x;
+                    }
+                    const uint32_t n_out = __shfl_sync(FULL_MASK, inc, 31), e_first = inc - n_f;
+                    const uint32_t has = __ballot_sync(FULL_MASK, n_f > 0);
+                    if (lane < 8) M.out_start[lane] = 0;
+                    __syncwarp();
+                    uint32_t to = 0;  // place of entry e of the output in the chunk's lists, minus e
+                    if (n_f) {
+                        const uint32_t at = atomicAdd(&M.q_list[owner], n_f) & 0xFFFFu;
+                        to = (uint32_t)(i0 + owner) * list_cap + at - e_first;
+                        atomicOr(&M.out_start[e_first >> 5], 1u << (e_first & 31u));
+                        M.out_lane[__popc(has & lt)] = (uint8_t)lane;
+                    }
+                    __syncwarp();
+                    uint32_t before = 0;
+                    for (uint32_t r = 0; r * 32 < n_out; ++r) {
+                        const uint32_t w = M.out_start[r];
+                        const uint32_t e = r * 32 + lane;
+                        const uint32_t src = M.out_lane[before + __popc(w & le) - 1];
+                        const uint32_t ef = __shfl_sync(FULL_MASK, e_first, src), d0 = __shfl_sync(FULL_MASK, to, src);
+                        if (e < n_out) glist[d0 + e] = M.found[(e - ef) * 32 + src];
+                        before += __popc(w);
+                    }
+                    __syncwarp();
+                }
+                if (locs) atomicAdd(&M.q_locs[owner], locs);
+                if (sect) atomicAdd(&M.q_sect[owner], sect);
+                // entry: lane | feature << 5; the step is the pair after home's
+                for (uint32_t step = 1; n_more; ++step) {
+                    __syncwarp();
+                    const uint32_t n_now = n_more;
+                    n_more = 0;
+                    for (uint32_t j0 = 0; j0 < n_now; j0 += 32) {
+                        const uint32_t en = j0 + lane < n_now ? M.more[j0 + lane] : 0u;
+                        bool over = true;
+                        const uint32_t h = M.hash[en];  // [feature * 32 + lane]
+                        const uint32_t home = tp.home(h);
+                        const uint32_t d = 2 * step - (home & 1u);  // of the pair's first word
+                        if (j0 + lane < n_now && d <= db.max_probe) {
+                            const uint32_t qi = M.item[r0 + (en & 31u)] >> 23;
+                            const ulonglong2 w =
+                                __ldcg(reinterpret_cast<const ulonglong2*>(db.table) + ((uint64_t)(home >> 1) + step));
+                            uint64_t e = w.x;
+                            uint32_t what = tp.step(e, d, h);
+                            if (what == 2 && d + 1 <= db.max_probe) {
+                                e = w.y;
+                                what = tp.step(e, d + 1, h);
+                            }
+                            if (what == 1) {
+                                const uint64_t bk = tp.bucket(e);
+                                const uint32_t at = atomicAdd(&M.q_list[qi], 1u) & 0xFFFFu;
+                                glist[(uint32_t)(i0 + qi) * list_cap + at] = bk;
+                                atomicAdd(&M.q_locs[qi], (uint32_t)bk & 0xFFFFu);
+                                if (Q.counters) atomicAdd(&M.q_sect[qi], sectors(bk));
+                            }
+                            over = what != 2;
+                        }
+                        __syncwarp();  // the entries are read before their places are taken again
+                        queue(!over, en);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        __syncwarp();
+        if (active) {
+            const uint32_t nm = in.m1 - in.m0;
+            const uint32_t sp = nm <= 1 ? span : max(span, Q.max_insert);
+            const uint32_t sws = sp >= k ? (sp - k + p.stride - 1) / p.stride + 1 : 0u;
+            const uint32_t lf = M.q_list[lane];
+            meta[i] = make_uint4(lf & 0xFFFFu, sws | ((lf >> 16) << META_FEAT_SHIFT), M.q_locs[lane], M.q_sect[lane]);
+        }
+        __syncwarp();
+    }
+}
+
 // Main path, part 2 (gather + score + label): one warp per query of the
 // chunk, KA histogram slots per warp in shared memory.  Queries whose
 // histogram does not fit are queued (chunk index) for the medium path.
@@ -884,21 +1237,23 @@ __global__ void __launch_bounds__(CLS_WARPS * 32, 8) k_classify_score(ClassifyDb
 }
 
 // Queries of the chunk with h_lo < H <= h_hi gathered locations (h_lo = 0:
-// no lower bound), not escalated: a warp takes groups of 32 consecutive
-// queries from a counter (*ctr, zero before the launch), reads their
-// metadata at once and takes those in range by ballot, so that warps that
-// start late take fewer groups.  With mid_list, the queries beyond h_hi
+// no lower bound), not escalated: a warp takes groups of 2^shift <= 32
+// consecutive queries from a counter (*ctr, zero before the launch), reads
+// their metadata at once and takes those in range by ballot, so that warps
+// that start late take fewer groups.  With mid_list, the queries beyond h_hi
 // are queued there (chunk index) as they are met.
 struct ChunkScan {
     uint32_t base, nq;  // first query of the current group, chunk size
+    uint32_t shift;     // log2 of the queries per group
     uint32_t* ctr;      // next group
     uint4 mt;           // this lane's query of the group
     uint32_t todo;      // lanes of the group still to be processed
 };
 
-__device__ __forceinline__ ChunkScan chunk_scan(uint32_t nq, uint32_t* ctr) {
+__device__ __forceinline__ ChunkScan chunk_scan(uint32_t nq, uint32_t shift, uint32_t* ctr) {
     ChunkScan it;
     it.nq = nq;
+    it.shift = shift;
     it.ctr = ctr;
     it.base = 0;
     it.todo = 0;
@@ -913,11 +1268,11 @@ __device__ __forceinline__ bool next_chunk_query(ChunkScan& it, const uint4* __r
         uint32_t g = 0;
         if (lane == 0) g = atomicAdd(it.ctr, 1u);
         g = __shfl_sync(FULL_MASK, g, 0);
-        const uint64_t first = (uint64_t)g * 32;
+        const uint64_t first = (uint64_t)g << it.shift;
         if (first >= it.nq) return false;
         it.base = (uint32_t)first;
         const uint64_t qi = first + lane;
-        it.mt = qi < it.nq ? meta[qi] : make_uint4(ESCALATED, 0, 0, 0);
+        it.mt = (lane >> it.shift) == 0 && qi < it.nq ? meta[qi] : make_uint4(ESCALATED, 0, 0, 0);
         const bool in = it.mt.x != ESCALATED && !(h_lo && it.mt.z <= h_lo);
         if (mid_list && in && it.mt.z > h_hi) mid_list[atomicAdd(mid_n, 1u)] = (uint32_t)qi;
         it.todo = __ballot_sync(FULL_MASK, in && it.mt.z <= h_hi);
@@ -998,15 +1353,39 @@ __global__ void __launch_bounds__(MED_WARPS * 32) k_classify_medium(ClassifyDb d
 }
 
 // ------------------------------------------------------------------
-// Sort path (databases with 32-bit locations): query steps 5-8 of
-// Section 5.2 for a query of at most 32*E gathered locations, on one warp,
-// by sorting instead of hashing.  The paper compacts the gathered locations
-// and sorts each read's segment (Sections 5.4-5.5); here one warp gathers
-// the query's locations straight into registers (E per lane, all loads in
-// flight at once), sorts them with an in-register bitonic network, and
-// reads off the window count statistic (runs of equal locations) and the
-// sliding-window scores (Section 5.6: elements in [x, x + sws) of the sorted
-// array) without a hash table.  Same outputs as query_score.
+// Sort path: query steps 5-8 of Section 5.2 for a query of at most 32*E
+// gathered locations, on one warp.  The paper compacts the gathered
+// locations and sorts each read's segment (Sections 5.4-5.5); here one warp
+// gathers the query's locations straight into registers (E per lane, all
+// loads in flight at once), drops those that cannot matter, and sorts the
+// rest with an in-register bitonic network to read off the window count
+// statistic (runs of equal locations) and the sliding-window scores
+// (Section 5.6: elements in [x, x + sws) of the sorted array).  Same outputs
+// as query_score.
+//
+// Dropping locations.  Windows are grouped into blocks of 2^b >= sws, so a
+// candidate's window range lies in its first window's block and the next
+// one.  Counting the locations per (target, block) in a small table
+// (colliding blocks share a counter, so a counter is never too low) bounds
+// the score of every candidate whose range can hold location X from above by
+// c(block of X) + max(c(block before), c(block after)).  With a threshold T,
+// every location that counts towards a candidate of score >= T has a bound
+// >= T; the others are dropped, and the scores of the candidates of score
+// >= T stay exact while all others stay below T.  T is guessed from the
+// largest bound; the guess is right if the top score s1 found this way puts
+// the close threshold (the smallest score that matters for the label) at T
+// or above, else the query is done once more with T = close(s1), which is
+// then right because the top score is at least s1.  With the full top-m list
+// requested the m-th score takes the place of the close threshold.
+//
+// What it saves, on 2 M pairs against the large database: of 495 locations
+// per query 96 are sorted (one query in 2,000 is done twice); the 512 and
+// 1024 classes take 3.30 and 3.23 ms against 4.96 and 7.28 ms with every
+// location sorted.  Half of that is the gather (about 45 G sectors/s, the
+// rate of random reads), the rest issue: about 1,500 warp instructions per
+// query.  More resident warps help more than the next query's gather in
+// flight behind the current one's sort (3.55 and 4.83 ms: its second buffer
+// costs a quarter of the warps).
 
 // Bitonic sort of 32*E keys held E per lane, element i = lane*E + r, into
 // ascending order of i.  Mirror form of the network: each merge stage of
@@ -1017,14 +1396,14 @@ __global__ void __launch_bounds__(MED_WARPS * 32) k_classify_medium(ClassifyDb d
 // registers; the stages beyond run as a loop whose body holds one mirror
 // step, the cross-lane half-cleaners (each guarded by the stage) and the
 // E/2 .. 1 in-register half-cleaners, which keeps the code small.
-template <int E>
-__device__ __forceinline__ void sort_in_lane_halves(uint32_t (&k)[E]) {
+template <int E, class T>
+__device__ __forceinline__ void sort_in_lane_halves(T (&k)[E]) {
 #pragma unroll
     for (int J = E >> 1; J > 0; J >>= 1) {
 #pragma unroll
         for (int r = 0; r < E; ++r) {
             if ((r & J) == 0) {
-                const uint32_t a = k[r], b = k[r | J];
+                const T a = k[r], b = k[r | J];
                 k[r] = min(a, b);
                 k[r | J] = max(a, b);
             }
@@ -1032,8 +1411,8 @@ __device__ __forceinline__ void sort_in_lane_halves(uint32_t (&k)[E]) {
     }
 }
 
-template <int E>
-__device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
+template <int E, class T>
+__device__ __forceinline__ void warp_bitonic_sort(T (&k)[E]) {
     const uint32_t lane = lane_id();
 #pragma unroll
     for (int K = 2; K <= E; K <<= 1) {
@@ -1041,7 +1420,7 @@ __device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
         for (int r = 0; r < E; ++r) {
             if ((r & (K >> 1)) == 0) {
                 const int o = r ^ (K - 1);
-                const uint32_t a = k[r], b = k[o];
+                const T a = k[r], b = k[o];
                 k[r] = min(a, b);
                 k[o] = max(a, b);
             }
@@ -1051,7 +1430,7 @@ __device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
 #pragma unroll
             for (int r = 0; r < E; ++r) {
                 if ((r & J) == 0) {
-                    const uint32_t a = k[r], b = k[r | J];
+                    const T a = k[r], b = k[r | J];
                     k[r] = min(a, b);
                     k[r | J] = max(a, b);
                 }
@@ -1065,14 +1444,18 @@ __device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
             // E-1-r; the lower lane keeps the minimum.  As a mirror pair
             // (r, E-1-r) of this lane meets the pair (E-1-r, r) of the
             // partner, each register takes the partner's value first.
-            const uint32_t up = (lane & (kl >> 1)) ? 0xFFFFFFFFu : 0u;  // the upper lane keeps the max
+            const T up = (lane & (kl >> 1)) ? ~(T)0 : (T)0;  // the upper lane keeps the max
             const uint32_t lm = kl - 1;
+            if (E == 1) {
+                const T o = __shfl_xor_sync(FULL_MASK, k[0], lm);
+                k[0] = up ? max(k[0], o) : min(k[0], o);
+            }
 #pragma unroll
             for (int r = 0; r < E / 2; ++r) {
-                const uint32_t a = k[r], b = k[E - 1 - r];
-                const uint32_t pa = __shfl_xor_sync(FULL_MASK, b, lm);  // partner's E-1-r
-                const uint32_t pb = __shfl_xor_sync(FULL_MASK, a, lm);  // partner's r
-                const uint32_t na = min(a, pa), nb = min(b, pb);
+                const T a = k[r], b = k[E - 1 - r];
+                const T pa = __shfl_xor_sync(FULL_MASK, b, lm);  // partner's E-1-r
+                const T pb = __shfl_xor_sync(FULL_MASK, a, lm);  // partner's r
+                const T na = min(a, pa), nb = min(b, pb);
                 k[r] = na ^ ((na ^ max(a, pa)) & up);
                 k[E - 1 - r] = nb ^ ((nb ^ max(b, pb)) & up);
             }
@@ -1081,11 +1464,11 @@ __device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
         for (int t = 3; t >= 0; --t) {  // lane distances kl/4 .. 1 (warp-uniform guard)
             const uint32_t lj = 1u << t;
             if (lj <= (kl >> 2)) {
-                const uint32_t up = (lane & lj) ? 0xFFFFFFFFu : 0u;
+                const T up = (lane & lj) ? ~(T)0 : (T)0;
 #pragma unroll
                 for (int r = 0; r < E; ++r) {
-                    const uint32_t o = __shfl_xor_sync(FULL_MASK, k[r], lj);
-                    const uint32_t n = min(k[r], o);
+                    const T o = __shfl_xor_sync(FULL_MASK, k[r], lj);
+                    const T n = min(k[r], o);
                     k[r] = n ^ ((n ^ max(k[r], o)) & up);
                 }
             }
@@ -1094,159 +1477,188 @@ __device__ __forceinline__ void warp_bitonic_sort(uint32_t (&k)[E]) {
     }
 }
 
-// Per-warp shared memory of the sort path: bucket list, its prefix, and per
-// run of equal locations in the sorted gather (at most 32*E runs) its
-// location, its first sorted index and its score.
-template <int E>
-__host__ __device__ constexpr size_t sort_warp_bytes(uint32_t list_cap) {
-    return align16((size_t)list_cap * 8) + align16(((size_t)list_cap + 4) * 4) + align16((32 * (size_t)E + 4) * 4) +
-           align16((32 * (size_t)E + 4) * 2) + align16((32 * (size_t)E) * 2);
-}
+constexpr int SORT_WARPS = 4;           // warps per CTA of the sort path
+constexpr int GU = 4;                   // gather steps unrolled together
+constexpr uint32_t SMALL_SORT = 256;    // survivors that are sorted eight per lane
+constexpr uint32_t NO_FILTER = 64;      // locations that are sorted without a look at the counts
 
-// Slot of loc[] and rs[] beyond every run (the arrays hold 32*E + 4).
-template <int E>
-constexpr uint32_t SORT_SPARE_SLOT = 32 * E + 3;
-
-struct SortWarpMem {
-    uint64_t* list;   // found buckets, offset << 16 | size
-    uint32_t* l_pre;  // exclusive prefix of the bucket sizes
-    uint32_t* loc;    // location of run j, ascending
-    uint16_t* rs;     // first sorted index of run j; rs[D] = H
-    uint16_t* sc;     // sliding-window score of run j (0 once excluded)
+// Per-warp shared memory of the sort path: the buckets' location indices,
+// the bitmap of bucket starts in the flat list, the gathered locations, and
+// three regions used in turn: `a` holds the
+// block counters (16 bits), then the sorted survivors and their runs'
+// locations; `b` the surviving locations, then the runs' first sorted indices
+// (rs); `c` the counter slots, then the bounds, then the runs' scores.  When
+// all the locations have to be sorted, they are so in place (raw) and `a`
+// takes rs.  The gathered locations stay here rather than in registers: the
+// loops over them then take H / 32 steps of a small body (unrolled over
+// registers, a query missed the instruction cache all the way).
+template <int E, class LocT>
+struct SortMem {
+    static constexpr uint32_t CAP = 32 * E;
+    static constexpr uint32_t SURV = CAP < SMALL_SORT ? CAP : SMALL_SORT;
+    static constexpr size_t BM_BYTES = align16((E + GU) * 4);
+    static constexpr size_t RAW_BYTES = align16((CAP + 4) * sizeof(LocT));
+    static constexpr size_t SURV_BYTES = align16(SURV * sizeof(LocT));
+    static constexpr size_t U16_BYTES = align16((CAP + 4) * 2);
+    static constexpr size_t A_BYTES = SURV_BYTES > U16_BYTES ? SURV_BYTES : U16_BYTES;
+    static constexpr size_t B_BYTES = align16((SURV + 4) * 2) > SURV_BYTES ? align16((SURV + 4) * 2) : SURV_BYTES;
+    uint64_t* adj;  // bucket b's first location minus its place in the flat list
+    uint32_t* bm;   // bit i of word r: element 32 r + i of the flat list starts a bucket
+    LocT* raw;      // the gathered locations, in the order of the flat list
+    unsigned char *a, *b;
+    uint16_t* c;
+    __host__ __device__ static constexpr size_t bytes(uint32_t list_cap) {
+        return align16((size_t)list_cap * 8) + BM_BYTES + RAW_BYTES + A_BYTES + B_BYTES + U16_BYTES;
+    }
+    __device__ __forceinline__ SortMem(unsigned char* p, uint32_t list_cap) {
+        adj = reinterpret_cast<uint64_t*>(p);
+        p += align16((size_t)list_cap * 8);
+        bm = reinterpret_cast<uint32_t*>(p);
+        p += BM_BYTES;
+        raw = reinterpret_cast<LocT*>(p);
+        p += RAW_BYTES;
+        a = p;
+        p += A_BYTES;
+        b = p;
+        p += B_BYTES;
+        c = reinterpret_cast<uint16_t*>(p);
+    }
+    // adds one to counter s; a counter never passes 32 E < 65,536
+    __device__ __forceinline__ void count(uint32_t s) const {
+        atomicAdd(reinterpret_cast<uint32_t*>(a) + (s >> 1), 1u << ((s & 1u) * 16));
+    }
 };
 
-template <int E>
-__device__ __forceinline__ SortWarpMem sort_warp_mem(unsigned char* p, uint32_t list_cap) {
-    SortWarpMem m;
-    m.list = reinterpret_cast<uint64_t*>(p);
-    p += align16((size_t)list_cap * 8);
-    m.l_pre = reinterpret_cast<uint32_t*>(p);
-    p += align16(((size_t)list_cap + 4) * 4);
-    m.loc = reinterpret_cast<uint32_t*>(p);
-    p += align16((32 * (size_t)E + 4) * 4);
-    m.rs = reinterpret_cast<uint16_t*>(p);
-    p += align16((32 * (size_t)E + 4) * 2);
-    m.sc = reinterpret_cast<uint16_t*>(p);
-    return m;
-}
-
-constexpr int SORT_WARPS = 4;  // warps per CTA of the sort path
-
-// First run index in [lo, hi) whose location is greater than v (hi if none).
-__device__ __forceinline__ uint32_t runs_upper_bound(const uint32_t* loc, uint32_t lo, uint32_t hi, uint32_t v) {
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (loc[mid] <= v) lo = mid + 1; else hi = mid;
+// The block counters' view of a location: 2^b >= sws windows per block, the
+// counters of a target's consecutive blocks next to each other.
+template <class LocT>
+struct BlockSlot {
+    uint32_t jb, jmask, b;
+    __device__ __forceinline__ uint32_t operator()(LocT x, uint32_t mask) const {
+        const uint32_t t = (uint32_t)(x >> jb);
+        return ((((uint32_t)x & jmask) >> b) + ((t * 0x9E3779B1u) >> 16)) & mask;
     }
-    return lo;
-}
+};
 
-// Sort path, step 1 of a query: copies its bucket list from src to working
-// memory and issues the loads of its H <= 32*E locations into k (element
-// x = r * 32 + lane of the flat location list; NO_LOC beyond H).
-constexpr uint32_t NO_LOC = 0xFFFFFFFFu;  // padding; sorts last and lies beyond H
-
-template <int E>
-__device__ __forceinline__ void sort_gather(const ClassifyDb& db, const SortWarpMem& M, const uint64_t* src,
-                                           uint32_t n_list, uint32_t H, uint32_t (&k)[E]) {
+// Starts gathering a query's H <= 32*E locations into M.raw: asynchronous
+// copies of one location each, so that all of them are in flight at once
+// without a register each (completion: cp_async_wait_all).  The bucket of an
+// element is the number of bucket starts up to it, read off the bitmap.
+template <int E, class LocT>
+__device__ __forceinline__ void sort_gather(const ClassifyDb& db, const SortMem<E, LocT>& M, const uint64_t* src,
+                                           uint32_t n_list, uint32_t H) {
     const uint32_t lane = lane_id();
-    const uint32_t* __restrict__ locs = static_cast<const uint32_t*>(db.locs);
-    uint64_t* list = M.list;
-    uint32_t* l_pre = M.l_pre;
-    __syncwarp();  // the previous query is done with the list
-    for (uint32_t j = lane; j < n_list; j += 32) list[j] = __ldg(src + j);
+    const LocT* __restrict__ locs = static_cast<const LocT*>(db.locs);
+    __syncwarp();  // the last query is done with the working memory
+#pragma unroll
+    for (int r = 0; r < E + GU; r += 32)
+        if (r + lane < E + GU) M.bm[r + lane] = 0;
     __syncwarp();
-
-    // exclusive prefix of the bucket sizes
     uint32_t tot = 0;
     for (uint32_t base = 0; base < n_list; base += 32) {
         const uint32_t idx = base + lane;
-        const uint32_t c = idx < n_list ? (uint32_t)(list[idx] & 0xFFFFu) : 0;
+        const uint64_t e = idx < n_list ? __ldg(src + idx) : 0;
+        const uint32_t c = (uint32_t)e & 0xFFFFu;
         uint32_t inc = c;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t x = __shfl_up_sync(FULL_MASK, inc, d);
             if ((int)lane >= d) inc += x;
         }
-        if (idx < n_list) l_pre[idx] = tot + inc - c;
+        if (idx < n_list) {
+            const uint32_t pre = tot + inc - c;
+            M.adj[idx] = (e >> 16) - pre;
+            atomicOr(&M.bm[pre >> 5], 1u << (pre & 31u));
+        }
         tot += __shfl_sync(FULL_MASK, inc, 31);
     }
-    if (lane == 0) l_pre[n_list] = tot;
     __syncwarp();
-
-    uint32_t lo = 0, hi = n_list;  // bucket of x = lane: last b with l_pre[b] <= lane
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (l_pre[mid] <= lane) lo = mid; else hi = mid;
-    }
-    uint32_t bkt = lo;
+    const uint32_t le = lanemask_lt() | (1u << lane);
+    uint32_t before = 0;
+#pragma unroll 1
+    for (uint32_t x0 = lane, r = 0; r * 32 < H; r += GU, x0 += 32 * GU) {
 #pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const uint32_t x = (uint32_t)r * 32 + lane;
-        k[r] = NO_LOC;
-        if (x < H) {
-            while (l_pre[bkt + 1] <= x) ++bkt;
-            k[r] = __ldg(locs + (list[bkt] >> 16) + (x - l_pre[bkt]));
+        for (int u = 0; u < GU; ++u) {
+            const uint32_t w = M.bm[r + u];
+            const uint32_t x = x0 + 32 * u;
+            if (x < H) {
+                const LocT* g = locs + (M.adj[before + __popc(w & le) - 1] + x);
+                const unsigned d = (unsigned)__cvta_generic_to_shared(M.raw + x);
+                if (sizeof(LocT) == 4)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(g) : "memory");
+                else
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(g) : "memory");
+            }
+            before += __popc(w);
         }
+    }
+    cp_async_commit();
+}
+
+// Sorts the n <= 32*EE locations src and leaves them ascending in dst.  A
+// function of its own for every size: a query runs one of them, and the
+// others do not lie between the steps before and after.
+template <int EE, class LocT>
+__device__ __noinline__ void sort_to(LocT* dst, const LocT* src, uint32_t n) {
+    const uint32_t lane = lane_id();
+    LocT k[EE];
+#pragma unroll
+    for (int r = 0; r < EE; ++r) {
+        const uint32_t x = (uint32_t)r * 32 + lane;
+        k[r] = x < n ? src[x] : ~(LocT)0;
+    }
+    warp_bitonic_sort<EE>(k);
+    __syncwarp();  // (dst may still be read as counters)
+    LocT* o = dst + lane * EE;
+#pragma unroll
+    for (int r = 0; r < EE; r += 2) {  // vector stores
+        if (EE == 1)
+            o[r] = k[r];
+        else if (sizeof(LocT) == 8)
+            *reinterpret_cast<ulonglong2*>(o + r) = make_ulonglong2((uint64_t)k[r], (uint64_t)k[(r + 1) % EE]);
+        else
+            *reinterpret_cast<uint2*>(o + r) = make_uint2((uint32_t)k[r], (uint32_t)k[(r + 1) % EE]);
     }
 }
 
-// Sort path, step 2 of a query: its H gathered locations k (as left by
-// sort_gather) are sorted, scored and labelled, and the outputs written.
-template <int E>
-__device__ __forceinline__ void query_sort(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
-                                          const SortWarpMem& M, uint32_t sws, uint32_t H, uint32_t (&k)[E],
-                                          Counters& ctr) {
+// Steps 5-8 of a query from its n locations, sorted in loc: runs, scores,
+// top m, label.  Locations may have been dropped with threshold T (see
+// above).  Returns 0 with the outputs written, or, if T turns out too high,
+// the threshold to use instead.
+// rs and score: working memory of n + 1 and n entries.
+template <class LocT>
+__device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q, LocT* loc,
+                                                 uint16_t* rs, uint16_t* score, uint32_t sws, uint32_t n, uint32_t T,
+                                                 uint32_t& distinct) {
     const uint32_t lane = lane_id();
-    const uint32_t jb = db.jbits;
-    warp_bitonic_sort<E>(k);
-
+    const uint32_t lt = lanemask_lt();
+    const uint32_t jb = sizeof(LocT) == 8 ? 32u : db.jbits;
+    const uint32_t jmask = sizeof(LocT) == 8 ? 0xFFFFFFFFu : (1u << jb) - 1u;
     // Runs of equal locations (the window count statistic of Section 5.6):
     // run j has location loc[j] and covers sorted indices [rs[j], rs[j+1]).
-    uint32_t D;
-    {
-        // bit r of starts: element lane*E + r (< H) begins a run
-        using Mask = typename std::conditional<(E > 32), unsigned long long, uint32_t>::type;
-        constexpr int MB = 8 * (int)sizeof(Mask);
-        const uint32_t before = __shfl_up_sync(FULL_MASK, k[E - 1], 1);
-        Mask starts = 0;
-#pragma unroll
-        for (int r = 0; r < E; ++r) starts |= (Mask)(k[r] != (r ? k[r - 1] : before)) << r;
-        const uint32_t first = lane * E;
-        const uint32_t valid = H > first ? min((uint32_t)E, H - first) : 0u;
-        starts &= valid >= (uint32_t)MB ? ~(Mask)0 : (((Mask)1 << valid) - 1);
-        if (lane == 0 && H > 0) starts |= 1;
-        const uint32_t n = (uint32_t)(MB == 64 ? __popcll((unsigned long long)starts) : __popc((uint32_t)starts));
-        uint32_t inc = n;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t x = __shfl_up_sync(FULL_MASK, inc, d);
-            if ((int)lane >= d) inc += x;
+    // Written over the sorted locations: a run's index is at most its first
+    // element's, and a round's elements are read before its runs are written.
+    uint32_t D = 0;
+    LocT carry = 0;  // the element before the round's first
+    for (uint32_t base = 0; base < n; base += 32) {
+        const uint32_t i = base + lane;
+        const LocT x = i < n ? loc[i] : (LocT)0;
+        LocT prev = __shfl_up_sync(FULL_MASK, x, 1);
+        if (lane == 0) prev = carry;
+        carry = __shfl_sync(FULL_MASK, x, 31);
+        const bool start = i < n && (i == 0 || x != prev);
+        const uint32_t b = __ballot_sync(FULL_MASK, start);
+        if (start) {
+            const uint32_t pos = D + __popc(b & lt);
+            loc[pos] = x;
+            rs[pos] = (uint16_t)i;
         }
-        D = __shfl_sync(FULL_MASK, inc, 31);
-        // the run starts in order (for E = 32 the other elements write to a
-        // spare slot instead of being predicated off, which keeps the
-        // kernel's predicate registers within what the compiler can allocate)
-        uint32_t pos = inc - n;
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const uint32_t b = (uint32_t)(starts >> r) & 1u;
-            if (E >= 32) {
-                const uint32_t at = b ? pos : SORT_SPARE_SLOT<E>;
-                M.loc[at] = k[r];
-                M.rs[at] = (uint16_t)(lane * E + r);
-            } else if (b) {
-                M.loc[pos] = k[r];
-                M.rs[pos] = (uint16_t)(lane * E + r);
-            }
-            pos += b;
-        }
+        D += __popc(b);
         __syncwarp();
-        if (lane == 0) M.rs[D] = (uint16_t)H;
     }
+    if (lane == 0) rs[D] = (uint16_t)n;
     __syncwarp();
-    ctr.locations += H;
-    ctr.distinct += D;
+    distinct = D;
 
     // Sliding-window scores (Section 5.6): the score of run j is the number
     // of sorted locations in [loc[j], hi], hi = loc[j] + sws - 1 cut at the
@@ -1255,23 +1667,23 @@ __device__ __forceinline__ void query_sort(const ClassifyDb& db, const ClassifyQ
     // and the score is rs[e] - rs[j].  Four runs are checked per step (the
     // locations ascend, so the count of those <= hi is the advance).  The
     // first top-m round is folded in.
-    const uint32_t jmask = (1u << jb) - 1u;
     const uint32_t w1 = sws ? sws - 1 : 0u;  // no wrap: stays in the run's target
     Cand best = Cand{0, 0xFFFFFFFFu, 0xFFFFFFFFu, 0};
     for (uint32_t j = lane; j < D; j += 32) {
-        const uint32_t x = M.loc[j];
-        const uint32_t hi = x + min(w1, jmask - (x & jmask));
+        const LocT x = loc[j];
+        const uint32_t win = (uint32_t)x & jmask;
+        const LocT hi = x + min(w1, jmask - win);
         uint32_t e = j + 1;
         for (;;) {
             uint32_t adv = 0;
 #pragma unroll
-            for (int d = 0; d < 4; ++d) adv += (e + d < D && M.loc[e + d] <= hi) ? 1u : 0u;
+            for (int d = 0; d < 4; ++d) adv += (e + d < D && loc[e + d] <= hi) ? 1u : 0u;
             e += adv;
             if (adv < 4) break;
         }
-        const uint32_t sc = (uint32_t)M.rs[e] - (uint32_t)M.rs[j];
-        M.sc[j] = (uint16_t)sc;
-        const Cand c = Cand{sc, x >> jb, x & jmask, 0};
+        const uint32_t sc = (uint32_t)rs[e] - (uint32_t)rs[j];
+        score[j] = (uint16_t)sc;
+        const Cand c = Cand{sc, (uint32_t)(x >> jb), win, 0};
         if (better(c, best)) best = c;
     }
     __syncwarp();
@@ -1291,15 +1703,15 @@ __device__ __forceinline__ void query_sort(const ClassifyDb& db, const ClassifyQ
         if (rd) {
             best = Cand{0, 0xFFFFFFFFu, 0xFFFFFFFFu, 0};
             for (uint32_t j = lane; j < D; j += 32) {
-                const uint32_t sc = M.sc[j];
+                const uint32_t sc = score[j];
                 if (sc == 0) continue;
-                const uint32_t x = M.loc[j];
-                const uint32_t t = x >> jb;
+                const LocT x = loc[j];
+                const uint32_t t = (uint32_t)(x >> jb);
                 if (t == prev_t) {
-                    M.sc[j] = 0;
+                    score[j] = 0;
                     continue;
                 }
-                const Cand c = Cand{sc, t, x & jmask, 0};
+                const Cand c = Cand{sc, t, (uint32_t)x & jmask, 0};
                 if (better(c, best)) best = c;
             }
         }
@@ -1310,27 +1722,32 @@ __device__ __forceinline__ void query_sort(const ClassifyDb& db, const ClassifyQ
                 __reduce_min_sync(FULL_MASK, (best.score == ms && best.t == mt) ? best.j0 : 0xFFFFFFFFu);
             best = Cand{ms, mt, mj, 0};
         }
+        if (Q.cands && best.score < T && T > 1) return 1;  // the full list needs every location
         if (best.score == 0) break;
         prev_t = best.t;
         if (Q.cands) {
             // last window of the range present: the location of the last run <= hi
-            const uint32_t x0 = (best.t << jb) | best.j0;
-            const uint32_t hi = x0 + min(w1, jmask - best.j0);
-            const uint32_t e = runs_upper_bound(M.loc, 0, D, hi);
-            best.j1 = M.loc[e - 1] & jmask;
+            const LocT x0 = ((LocT)best.t << jb) | best.j0;
+            const LocT hi = x0 + min(w1, jmask - best.j0);
+            uint32_t lo = 0, up = D;  // first run beyond hi
+            while (lo < up) {
+                const uint32_t mid = (lo + up) >> 1;
+                if (loc[mid] <= hi) lo = mid + 1; else up = mid;
+            }
+            best.j1 = (uint32_t)loc[lo - 1] & jmask;
         }
         if ((int)lane == rd) mine = best;
         if (rd == 0) {
             hits = best.score;
             top = best.t;
             bar = (uint64_t)(100 - Q.band) * hits;
+            const uint32_t s_min = (uint32_t)((bar + 99) / 100);  // smallest score s with 100 s >= bar
+            if (!Q.cands && s_min < T && T > 1) return max(s_min, 1u);
             if (hits >= Q.hits_min) label = top < db.n_targets ? db.taxon_of_target[top] : NO_TAXON;
             else if (!Q.cands) break;
             if (!Q.cands) {
-                // smallest score s with 100 s >= bar
-                const uint32_t s_min = (uint32_t)((bar + 99) / 100);
                 for (uint32_t j = lane; j < D; j += 32)
-                    if (M.sc[j] < s_min) M.sc[j] = 0;
+                    if (score[j] < s_min) score[j] = 0;
             }
         } else if (hits >= Q.hits_min && 100ull * best.score >= bar) {
             const uint32_t tx = best.t < db.n_targets ? db.taxon_of_target[best.t] : NO_TAXON;
@@ -1341,43 +1758,140 @@ __device__ __forceinline__ void query_sort(const ClassifyDb& db, const ClassifyQ
         __syncwarp();
     }
     write_result(Q, q, label, hits, top, mine);
+    return 0;
+}
+
+// One query of H <= 32*E locations, gathered in M.raw.  Returns false if its
+// survivors do not fit the small sorts and there is no sort of all the
+// locations (64-bit locations): the query goes to the medium path.
+template <int E, class LocT>
+__device__ __forceinline__ bool query_sort(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+                                          const SortMem<E, LocT>& M, uint32_t sws, uint32_t H,
+                                          uint32_t& distinct) {
+    using Mem = SortMem<E, LocT>;
+    constexpr uint32_t MASK = Mem::CAP - 1;  // block counters
+    const uint32_t lane = lane_id();
+    const uint32_t lt = lanemask_lt();
+    BlockSlot<LocT> bs;
+    bs.jb = sizeof(LocT) == 8 ? 32u : db.jbits;
+    bs.jmask = sizeof(LocT) == 8 ? 0xFFFFFFFFu : (1u << bs.jb) - 1u;
+    bs.b = sws > 1 ? 32u - (uint32_t)__clz(sws - 1) : 0u;  // 2^b >= sws (sws < 2^17)
+    const uint16_t* cnt = reinterpret_cast<const uint16_t*>(M.a);
+    LocT* const raw = M.raw;
+    LocT* surv = reinterpret_cast<LocT*>(M.b);
+    // the counters of mc_classify_debug count all distinct locations
+    uint32_t T = (H <= NO_FILTER || Q.counters) ? 1u : 0u;
+    do {
+        const LocT* from = raw;
+        uint32_t n = H;
+        if (T != 1) {
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < E / 8; ++i) reinterpret_cast<uint4*>(M.a)[i * 32 + lane] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+#pragma unroll 2
+            for (uint32_t x = lane; x < H; x += 32) {
+                const uint32_t s = bs(raw[x], MASK);
+                M.c[x] = (uint16_t)s;
+                M.count(s);
+            }
+            __syncwarp();
+            uint32_t most = 0;
+#pragma unroll 2
+            for (uint32_t x = lane; x < H; x += 32) {
+                const uint32_t s = M.c[x];
+                const uint32_t u = (uint32_t)cnt[s] + max(cnt[(s - 1) & MASK], cnt[(s + 1) & MASK]);
+                most = max(most, u);
+                M.c[x] = (uint16_t)u;
+            }
+            if (T == 0) {
+                // aim a little below the close threshold of the largest
+                // bound (for a full list, at a quarter of it), as the top
+                // score may be lower than its bound
+                most = __reduce_max_sync(FULL_MASK, most);
+                const uint32_t close = ((100 - Q.band) * most + 99) / 100;
+                T = max(Q.cands ? most / 4 : close - close / 8, 1u);
+            }
+            n = 0;
+#pragma unroll 2
+            for (uint32_t x0 = 0; x0 < H; x0 += 32) {
+                const uint32_t x = x0 + lane;
+                const bool in = x < H && M.c[x] >= T;
+                const uint32_t v = __ballot_sync(FULL_MASK, in);
+                const uint32_t at = n + __popc(v & lt);
+                if (in && at < Mem::SURV) surv[at] = raw[x];
+                n += __popc(v);
+            }
+            from = surv;
+        }
+        __syncwarp();
+        LocT* loc = reinterpret_cast<LocT*>(M.a);
+        uint16_t* rs = reinterpret_cast<uint16_t*>(M.b);
+        if (n <= 32) {
+            sort_to<1>(loc, from, n);
+        } else if (n <= 64) {
+            sort_to<2>(loc, from, n);
+        } else if (n <= 128) {
+            sort_to<4>(loc, from, n);
+        } else if (E <= 8 || n <= SMALL_SORT) {
+            sort_to<8>(loc, from, n);
+        } else if (sizeof(LocT) == 4) {
+            n = H;  // too many left: sort them all, in place
+            T = 1;
+            loc = raw;
+            rs = reinterpret_cast<uint16_t*>(M.a);
+            sort_to<E>(loc, (const LocT*)raw, n);
+        } else {
+            return false;
+        }
+        __syncwarp();
+        T = score_sorted<LocT>(db, Q, q, loc, rs, M.c, sws, n, T, distinct);
+    } while (T != 0);
+    return true;
 }
 
 // Resident CTAs per SM that the register budget of a sort-path kernel is
-// sized for (shared memory admits 15, 10, 5 and 3 for E = 8, 16, 32, 64).
-template <int E>
-constexpr int sort_min_ctas() { return E == 8 ? 8 : (E == 16 ? 7 : (E == 32 ? 5 : 3)); }
+// sized for.
+template <int E, class LocT>
+constexpr int sort_min_ctas() {
+    return sizeof(LocT) == 8 ? (E == 8 ? 5 : (E == 16 ? 4 : 2)) : (E == 8 ? 8 : (E == 16 ? 8 : (E == 32 ? 5 : 3)));
+}
 
 // Sort path over the chunk's queries with h_lo < H <= 32*E gathered
-// locations; with mid_list (the largest class), larger ones are queued for
-// the medium path.
-template <int E>
-__global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E>()) k_classify_sort(ClassifyDb db, ClassifyQuery Q, uint32_t q0,
-                                                                  uint32_t chunk, uint32_t list_cap,
-                                                                  const uint64_t* __restrict__ glist,
-                                                                  const uint4* __restrict__ meta, uint32_t h_lo,
-                                                                  uint32_t* __restrict__ mid_list,
-                                                                  uint32_t* __restrict__ mid_n,
-                                                                  uint32_t* __restrict__ group_ctr) {
+// locations; with last (the largest class), larger ones are queued for the
+// medium path.
+template <int E, class LocT>
+__global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
+    k_classify_sort(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t chunk, uint32_t list_cap,
+                    const uint64_t* __restrict__ glist, const uint4* __restrict__ meta, uint32_t h_lo, bool last,
+                    uint32_t group_shift, uint32_t* __restrict__ mid_list, uint32_t* __restrict__ mid_n,
+                    uint32_t* __restrict__ group_ctr) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t w = threadIdx.x >> 5;
-    const SortWarpMem M = sort_warp_mem<E>(smem + w * sort_warp_bytes<E>(list_cap), list_cap);
-    Counters ctr;
+    const SortMem<E, LocT> M(smem + w * SortMem<E, LocT>::bytes(list_cap), list_cap);
     const uint32_t total = total_queries(Q);
     if (q0 < total) {
-        ChunkScan it = chunk_scan(min(chunk, total - q0), group_ctr);
+        ChunkScan it = chunk_scan(min(chunk, total - q0), group_shift, group_ctr);
         uint32_t i;
         uint4 mt;
-        uint32_t k[E];
-        while (next_chunk_query(it, meta, h_lo, 32u * E, mid_list, mid_n, i, mt)) {
-            sort_gather<E>(db, M, glist + (uint64_t)i * list_cap, mt.x, mt.z, k);
-            query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, k, ctr);
-            ctr.features += meta_feat(mt);
-            ctr.found += mt.x;
-            ctr.sectors += mt.w;
-            ++ctr.queries;
+        while (next_chunk_query(it, meta, h_lo, 32u * E, last ? mid_list : nullptr, mid_n, i, mt)) {
+            sort_gather<E>(db, M, glist + (uint64_t)i * list_cap, mt.x, mt.z);
+            cp_async_wait_all();
+            __syncwarp();
+            uint32_t distinct;
+            if (!query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct)) {
+                if (lane_id() == 0) mid_list[atomicAdd(mid_n, 1u)] = i;
+            } else if (Q.counters) {  // per query: a debug call need not keep them in registers
+                Counters ctr;
+                ctr.features = meta_feat(mt);
+                ctr.locations = mt.z;
+                ctr.distinct = distinct;
+                ctr.found = mt.x;
+                ctr.sectors = mt.w;
+                ctr.queries = 1;
+                flush_counters(Q, ctr, E == 8 ? 1 : (E == 16 ? 2 : (E == 32 ? 3 : 6)));
+            }
         }
-        flush_counters(Q, ctr, E == 8 ? 1 : (E == 16 ? 2 : (E == 32 ? 3 : 6)));
     }
     // Launched as a programmatic dependent of the medium path, this kernel
     // may run alongside it; waiting for that grid before exiting makes this
@@ -1431,6 +1945,26 @@ using LargeKernel = void (*)(ClassifyDb, ClassifyQuery, const uint32_t*, const u
                              size_t);
 using MediumKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, const uint64_t*, const uint4*,
                               const uint32_t*, const uint32_t*, uint32_t*, uint32_t*, uint32_t*);
+
+using LookupLanesKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint32_t, uint64_t*, uint4*,
+                                   uint32_t*, uint32_t*, uint32_t);
+
+template <int R, int KC>
+LookupLanesKernel lookup_lanes_for_lb(uint32_t lb) {
+    if (lb == 2) return k_lookup_lanes<R, KC, 2>;
+    if (lb == 8) return k_lookup_lanes<R, KC, 8>;
+    return k_lookup_lanes<R, KC, 4>;
+}
+
+// One window per lane (sketch sizes up to 16), or nullptr.
+LookupLanesKernel pick_lookup_lanes(const SketchParams& sp, uint32_t lb) {
+    if (sp.s > LS_MAX_S) return nullptr;
+    const int r = sketch_r_for(sp.w);
+    const bool k16 = sp.k == 16;
+    if (r == 4) return k16 ? lookup_lanes_for_lb<4, 16>(lb) : lookup_lanes_for_lb<4, 0>(lb);
+    if (r == 8) return k16 ? lookup_lanes_for_lb<8, 16>(lb) : lookup_lanes_for_lb<8, 0>(lb);
+    return k16 ? lookup_lanes_for_lb<16, 16>(lb) : lookup_lanes_for_lb<16, 0>(lb);
+}
 
 template <int R, int KC>
 LookupKernel lookup_for_lb(uint32_t lb) {
@@ -1498,15 +2032,24 @@ LargeKernel pick_large(const ClassifyDb& db) {
 
 // Kernels and launch shapes of one launch set.
 using SortKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint32_t, const uint64_t*, const uint4*,
-                            uint32_t, uint32_t*, uint32_t*, uint32_t*);
+                            uint32_t, bool, uint32_t, uint32_t*, uint32_t*, uint32_t*);
 
 // The sort path's size classes: queries of up to 256, 512, 1024 and 2048
 // gathered locations, each with its own kernel (E = 8, 16, 32, 64 per lane).
 constexpr int N_SORT_CLASSES = 4;
 constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {256, 512, 1024, 2048};
 
+// Launches of at least this many queries look up with one window per lane,
+// nine queries for each of the 3,648 resident warps; with fewer, lanes stay
+// empty and one warp per query is faster.  Measured (us, per query / per
+// lane): single reads of 100, 20,000 queries 41 / 58, 50,000 90 / 77; half
+// pairs, lengths 50-300, 20,000 queries 73 / 79, 50,000 147 / 130.
+constexpr uint32_t LANES_MIN_QUERIES = 32768;
+
 struct Geometry {
-    LookupKernel kl;
+    LookupKernel kl;         // one window per warp
+    LookupLanesKernel kll;   // one window per lane
+    uint32_t batch_shift;    // log2 of the queries a lookup warp takes at a time (kll)
     ScoreKernel ks;
     MediumKernel km;
     LargeKernel kb;
@@ -1516,6 +2059,7 @@ struct Geometry {
     uint32_t list_cap;
     size_t smem_l, smem_s, smem_m, per_warp_b, smem_t[N_SORT_CLASSES];
     uint32_t threads_l, threads_s, grid_l, grid_s, grid_m, blocks_b, grid_t[N_SORT_CLASSES];
+    uint32_t group_shift;  // log2 of the queries a sort-path warp takes at a time
 };
 
 cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratch& sc, Geometry* g) {
@@ -1524,7 +2068,9 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     g->list_cap = WIN_A * db.sp.s;
-    g->kl = pick_lookup(db.sp, t.probe_batch);
+    g->kll = sc.chunk >= LANES_MIN_QUERIES ? pick_lookup_lanes(db.sp, t.probe_batch) : nullptr;
+    g->kl = g->kll ? nullptr : pick_lookup(db.sp, t.probe_batch);
+    const void* const kl_any = g->kll ? (const void*)g->kll : (const void*)g->kl;
     const KeyMode km = key_mode(db, t);
     const bool compact = km == KeyMode::compact;
     g->ks = pick_score(t.hist_slots, t.gather_batch, km);
@@ -1540,15 +2086,15 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->grid_m = (uint32_t)sms * (uint32_t)std::max(occ_m, 1);
     g->threads_l = t.lookup_warps * 32;
     g->threads_s = t.score_warps * 32;
-    g->smem_l = t.lookup_warps * lookup_warp_bytes(g->list_cap);
+    g->smem_l = t.lookup_warps * (g->kll ? sizeof(LookupLanesMem) : lookup_warp_bytes(g->list_cap));
     g->smem_s = t.score_warps * (compact ? scratch_bytes<uint16_t, uint32_t>(t.hist_slots, g->list_cap, 0, 0)
                                          : scratch_bytes<uint16_t, uint64_t>(t.hist_slots, g->list_cap, 0, 0));
-    if ((e = cudaFuncSetAttribute(g->kl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_l)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(kl_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_l)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(g->ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_s)) != cudaSuccess)
         return e;
     int occ_l = 1, occ_s = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_l, g->kl, g->threads_l, g->smem_l)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_l, kl_any, g->threads_l, g->smem_l)) != cudaSuccess)
         return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, g->ks, g->threads_s, g->smem_s)) != cudaSuccess)
         return e;
@@ -1556,18 +2102,39 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     occ_s = std::max(occ_s, 1);
     const uint64_t c = std::max<uint32_t>(sc.chunk, 1);
     g->grid_l = (uint32_t)std::min<uint64_t>((c + t.lookup_warps - 1) / t.lookup_warps, (uint64_t)sms * occ_l);
+    g->batch_shift = 0;
+    if (g->kll) {
+        // a lane per query where that still gives every resident warp some
+        const uint64_t warps = (uint64_t)sms * occ_l * t.lookup_warps;
+        while (g->batch_shift < 5 && (c >> (g->batch_shift + 1)) >= warps) ++g->batch_shift;
+        const uint64_t batches = (c + (1u << g->batch_shift) - 1) >> g->batch_shift;
+        g->grid_l = (uint32_t)std::min<uint64_t>((batches + t.lookup_warps - 1) / t.lookup_warps, (uint64_t)sms * occ_l);
+    }
     g->grid_s = (uint32_t)std::min<uint64_t>((c + t.score_warps - 1) / t.score_warps, (uint64_t)sms * occ_s);
     g->per_warp_b = scratch_bytes<uint32_t>(KB_SLOTS, LIST_B, LIST_B, BUF_B);
     g->blocks_b = std::max<uint32_t>(1, sc.large_warps / CLS_WARPS);
-    // sort path: only for 32-bit locations with compact keys
-    g->sort = compact && t.score_mode != SCORE_HASH;
+    // sort path: locations sorted as they are stored (not with wide keys of 32-bit ones)
+    g->sort = km != KeyMode::wide32 && t.score_mode != SCORE_HASH;
     g->n_sort = 0;
+    g->group_shift = 0;
     if (g->sort) {
-        const SortKernel kts[N_SORT_CLASSES] = {k_classify_sort<8>, k_classify_sort<16>, k_classify_sort<32>,
-                                                k_classify_sort<64>};
-        const size_t bytes[N_SORT_CLASSES] = {sort_warp_bytes<8>(g->list_cap), sort_warp_bytes<16>(g->list_cap),
-                                              sort_warp_bytes<32>(g->list_cap), sort_warp_bytes<64>(g->list_cap)};
-        for (int c2 = 0; c2 < N_SORT_CLASSES && SORT_CLASS_MAX[c2] <= t.sort_max; ++c2) {
+        const SortKernel kts[N_SORT_CLASSES] = {
+            compact ? k_classify_sort<8, uint32_t> : k_classify_sort<8, uint64_t>,
+            compact ? k_classify_sort<16, uint32_t> : k_classify_sort<16, uint64_t>,
+            compact ? k_classify_sort<32, uint32_t> : k_classify_sort<32, uint64_t>,
+            compact ? k_classify_sort<64, uint32_t> : nullptr};
+        const uint32_t lc = g->list_cap;
+        const size_t bytes[N_SORT_CLASSES] = {
+            compact ? SortMem<8, uint32_t>::bytes(lc) : SortMem<8, uint64_t>::bytes(lc),
+            compact ? SortMem<16, uint32_t>::bytes(lc) : SortMem<16, uint64_t>::bytes(lc),
+            compact ? SortMem<32, uint32_t>::bytes(lc) : SortMem<32, uint64_t>::bytes(lc),
+            compact ? SortMem<64, uint32_t>::bytes(lc) : 0};
+        const uint32_t largest = compact ? t.sort_max : std::min(t.sort_max, 1024u);  // 64-bit keys: registers
+        // groups of 32 queries where every resident warp gets several,
+        // smaller ones in small launches, down to one query per warp
+        const uint64_t warps = (uint64_t)sms * 28;
+        while (g->group_shift < 5 && (c >> (g->group_shift + 1)) >= 4 * warps) ++g->group_shift;
+        for (int c2 = 0; c2 < N_SORT_CLASSES && SORT_CLASS_MAX[c2] <= largest; ++c2) {
             g->kt[c2] = kts[c2];
             g->smem_t[c2] = SORT_WARPS * bytes[c2];
             if ((e = cudaFuncSetAttribute(kts[c2], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_t[c2])) !=
@@ -1616,7 +2183,12 @@ uint32_t* queue_counters(const ClassifyScratch& sc) { return sc.ovf + sc.n_q_cap
 
 cudaError_t launch_lookup(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
                           uint32_t q0, cudaStream_t s) {
-    MC_LAUNCH("classify_lookup", s,
+    if (g.kll)
+        MC_LAUNCH("classify_lookup", s,
+                  g.kll<<<g.grid_l, g.threads_l, g.smem_l, s>>>(db, Q, q0, sc.chunk, g.list_cap, sc.glist, sc.meta,
+                                                               sc.ovf, queue_counters(sc), g.batch_shift));
+    else
+        MC_LAUNCH("classify_lookup", s,
               g.kl<<<g.grid_l, g.threads_l, g.smem_l, s>>>(db, Q, q0, sc.chunk, g.list_cap, sc.glist, sc.meta, sc.ovf,
                                                           queue_counters(sc)));
     return cudaGetLastError();
@@ -1632,15 +2204,16 @@ cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const Classif
     return cudaGetLastError();
 }
 
-// Score of the chunk at q0.  Sort path: the largest size class first (it
-// queues the queries beyond it), then the medium path, then the other
-// classes, the most populous one (512) launched with programmatic stream
-// serialization so that it fills the SMs the medium path's few long
+// Score of the chunk at q0.  Sort path, 32-bit locations: the largest size
+// class first (it queues the queries beyond it), then the medium path, then
+// the other classes, the most populous one (512) launched with programmatic
+// stream serialization so that it fills the SMs the medium path's few long
 // queries leave idle (they share no data: the sort kernels read the
 // lookup's outputs and write other queries' results; their groups of
 // queries come from a counter, so the CTAs that start late take fewer).
-// Hash path: the score kernel, then the medium path for the queries whose
-// histogram did not fit.
+// 64-bit locations: every class may queue queries, so the medium path comes
+// last.  Hash path: the score kernel, then the medium path for the queries
+// whose histogram did not fit.
 cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
                          uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
@@ -1657,13 +2230,15 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
     static const char* const names[N_SORT_CLASSES] = {"classify_sort256", "classify_sort512", "classify_sort1024",
                                                       "classify_sort2048"};
     const int last = g.n_sort - 1;
-    const int pdl = last >= 2 ? 1 : -1;  // the class launched as the medium path's dependent
+    const bool narrow = db.jbits != 0;
+    const int pdl = narrow && last >= 2 ? 1 : -1;  // the class launched as the medium path's dependent
     int order[N_SORT_CLASSES + 1], n = 0;
     order[n++] = last;
-    order[n++] = -1;  // medium path
+    if (narrow) order[n++] = -1;  // medium path
     if (pdl >= 0) order[n++] = pdl;
     for (int c = 0; c < last; ++c)
         if (c != pdl) order[n++] = c;
+    if (!narrow) order[n++] = -1;
     for (int k = 0; k < n; ++k) {
         const int c = order[k];
         if (c < 0) {
@@ -1681,11 +2256,10 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = c == pdl ? 1 : 0;
-        uint32_t* ml = c == last ? sc.mid : nullptr;
-        uint32_t* mn = c == last ? qc + 2 : nullptr;
         MC_LAUNCH(names[c], s,
                   e = cudaLaunchKernelEx(&cfg, g.kt[c], db, Q, q0, (uint32_t)sc.chunk, g.list_cap,
-                                         (const uint64_t*)sc.glist, (const uint4*)sc.meta, h_lo, ml, mn, qc + 5 + c));
+                                         (const uint64_t*)sc.glist, (const uint4*)sc.meta, h_lo, c == last, g.group_shift,
+                                         sc.mid, qc + 2, qc + 5 + c));
         if (e != cudaSuccess) return e;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1998,7 +2572,7 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
             }
         }
         // the sort path, for each largest size class
-        if (db.jbits) {
+        {
             for (uint32_t smax : {256u, 512u, 1024u, 2048u}) {
                 Tuning t = cur;
                 t.score_mode = SCORE_SORT;

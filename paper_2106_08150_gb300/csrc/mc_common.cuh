@@ -116,6 +116,34 @@ struct TableFmt {
     }
 };
 
+// A probe for h walks the words from its home slot on; d = slot - home.
+// The word's own home lies before, at or behind h's as its displacement is
+// above, equal to or below d, so the ordered probe needs no slot numbers:
+// the word's key is below h iff disp > d, or disp == d and its low bits are
+// below h's.  All fields lie in the word's low 32 bits or, for low, in 32
+// bits starting at cbits + TAB_DBITS <= 22.
+struct TableProbe {
+    uint32_t cbits, lbits, lmask;
+    __device__ __forceinline__ explicit TableProbe(const TableFmt& f)
+        : cbits(f.cbits), lbits(f.lbits()), lmask(f.lbits() ? 0xFFFFFFFFu >> (32 - f.lbits()) : 0u) {}
+    __device__ __forceinline__ uint32_t home(uint32_t h) const { return h >> lbits; }  // lbits <= 31
+    // 0: the word is empty or its key is above h (h is absent), 1: its key
+    // is h, 2: its key is below h (go on with the next word)
+    __device__ __forceinline__ uint32_t step(uint64_t e, uint32_t d, uint32_t h) const {
+        const uint32_t lo = (uint32_t)e, hi = (uint32_t)(e >> 32);
+        if ((lo & ((1u << cbits) - 1u)) == 0) return 0;
+        const uint32_t disp = (lo >> cbits) & TAB_MAX_DISP;
+        const uint32_t low = __funnelshift_r(lo, hi, cbits + TAB_DBITS) & lmask;
+        const uint32_t hl = h & lmask;
+        if (disp != d) return disp > d ? 2u : 0u;
+        return low == hl ? 1u : (low < hl ? 2u : 0u);
+    }
+    // bucket of a word, offset << 16 | count
+    __device__ __forceinline__ uint64_t bucket(uint64_t e) const {
+        return ((e >> (cbits + TAB_DBITS + lbits)) << 16) | ((uint32_t)e & ((1u << cbits) - 1u));
+    }
+};
+
 // Bits of the count field for a bucket cap.
 __host__ __device__ inline uint32_t count_bits(uint32_t cap) {
     uint32_t b = 1;

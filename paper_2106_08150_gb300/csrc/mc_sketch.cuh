@@ -19,6 +19,9 @@
 // windows can be sketched together so that their dependency chains overlap.
 #pragma once
 
+#include <type_traits>
+#include <utility>
+
 #include "mc_common.cuh"
 
 namespace mc {
@@ -337,26 +340,41 @@ __device__ __forceinline__ uint4 load_chunk(uintptr_t c, uintptr_t lo, uintptr_t
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Batcher's odd-even merge sort of 16 registers (63 comparators).
-__device__ __forceinline__ void sort16(uint32_t (&v)[16]) {
-#pragma unroll
-    for (int p = 1; p < 16; p <<= 1) {
-#pragma unroll
-        for (int k = p; k >= 1; k >>= 1) {
-#pragma unroll
-            for (int j = k % p; j + k < 16; j += 2 * k) {
-#pragma unroll
-                for (int i = 0; i < k; ++i) {
+// Batcher's odd-even merge sort of 16 registers: its 63 comparators as a
+// table, applied through a fold so that every register index is a constant
+// (left to loop unrolling, the compiler may give up and move the registers
+// to local memory).
+struct SortNet16 {
+    int a[63] = {}, b[63] = {};
+};
+constexpr SortNet16 make_sort_net16() {
+    SortNet16 n{};
+    int c = 0;
+    for (int p = 1; p < 16; p *= 2)
+        for (int k = p; k >= 1; k /= 2)
+            for (int j = k % p; j + k < 16; j += 2 * k)
+                for (int i = 0; i < k; ++i)
                     if (i + j + k < 16 && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
-                        const uint32_t a = v[i + j], b = v[i + j + k];
-                        v[i + j] = min(a, b);
-                        v[i + j + k] = max(a, b);
+                        n.a[c] = i + j;
+                        n.b[c++] = i + j + k;
                     }
-                }
-            }
-        }
-    }
+    return n;
 }
+
+__device__ __forceinline__ void compare_exchange(uint32_t& x, uint32_t& y) {
+    const uint32_t a = x, b = y;
+    x = min(a, b);
+    y = max(a, b);
+}
+
+template <size_t... I>
+__device__ __forceinline__ void sort16_steps(uint32_t (&v)[16], std::index_sequence<I...>) {
+    constexpr SortNet16 net = make_sort_net16();
+    (compare_exchange(v[std::integral_constant<int, net.a[I]>::value], v[std::integral_constant<int, net.b[I]>::value]),
+     ...);
+}
+
+__device__ __forceinline__ void sort16(uint32_t (&v)[16]) { sort16_steps(v, std::make_index_sequence<63>()); }
 
 // v = the 16 smallest of the sorted v and u, sorted.
 __device__ __forceinline__ void keep_smallest16(uint32_t (&v)[16], const uint32_t (&u)[16]) {
@@ -385,6 +403,19 @@ __device__ __forceinline__ void lane_candidate(uint32_t y, uint32_t tau, uint32_
         "@p add.u32 %0, %0, 128;\n\t}"
         : "+r"(at)
         : "r"(y), "r"(tau)
+        : "memory");
+}
+
+// The same if on is not 0.
+__device__ __forceinline__ void lane_candidate_if(uint32_t on, uint32_t y, uint32_t tau, uint32_t& at) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %3, 0;\n\t"
+        "setp.le.and.u32 p, %1, %2, q;\n\t"
+        "@p st.shared.u32 [%0], %1;\n\t"
+        "@p add.u32 %0, %0, 128;\n\t}"
+        : "+r"(at)
+        : "r"(y), "r"(tau), "r"(on)
         : "memory");
 }
 
@@ -459,21 +490,29 @@ __device__ __forceinline__ bool lane_sketch(const uint32_t* code, const uint16_t
                 }
             }
         } else {  // ends of sequences and windows, invalid bases
-            const uint32_t r_max = min(n_max - base, 16u);
-#pragma unroll 1
-            for (uint32_t r = 0; r < r_max; ++r) {
-                uint32_t f = __funnelshift_l(a1, a0, 2 * r);
-                uint32_t g = __funnelshift_r(r0, r1, 2 * r);
-                if (KC == 0) {
-                    f >>= 32 - 2 * k;
-                    g &= 0xFFFFFFFFu >> (32 - 2 * k);
+            const uint32_t r_max = n_max - base;
+#pragma unroll
+            for (int r4 = 0; r4 < 16; r4 += 4) {
+                if ((uint32_t)r4 < r_max) {
+#pragma unroll
+                    for (int r = r4; r < r4 + 4; ++r) {
+                        uint32_t f = __funnelshift_l(a1, a0, 2 * r);
+                        uint32_t g = __funnelshift_r(r0, r1, 2 * r);
+                        if (KC == 0) {
+                            f >>= 32 - 2 * k;
+                            g &= 0xFFFFFFFFu >> (32 - 2 * k);
+                        }
+                        lane_candidate_if(ok & (1u << (15 - r)), hash_h1_head(min(f, g)), tau, at);
+                    }
+                    if (r4 == 4 && at > col_cap) {
+                        over = true;
+                        at = col;
+                    }
                 }
-                const uint32_t y = hash_h1_head(min(f, g));
-                if ((ok >> (15 - r)) & 1u) lane_candidate(y, tau, at);
-                if (at > col_cap) {
-                    over = true;
-                    at = col;
-                }
+            }
+            if (at > col_cap) {
+                over = true;
+                at = col;
             }
         }
         a0 = a1;
