@@ -31,14 +31,13 @@ namespace mc {
 
 namespace {
 
-constexpr int CLS_WARPS = 4;                 // warps per CTA (score and large paths)
+constexpr int CLS_WARPS = 4;                 // warps per CTA (score path)
 constexpr int LK_WARPS = 8;                  // warps per CTA (lookup path)
 constexpr int WIN_A = 8;                     // windows per query on the shared-memory path
 constexpr uint32_t KB_SLOTS = 1u << 16;      // large-path histogram slots per warp
 constexpr uint32_t LIST_B = MC_MAX_QUERY_WINDOWS * MAX_S;
-constexpr int B_WARPS_PER_SM = 2;
-constexpr uint32_t KM_SLOTS = 2048;          // medium-path histogram slots per warp
-constexpr int MED_WARPS = 2;                 // warps per CTA (medium path)
+constexpr int B_WARPS_PER_SM = 2;  // large-path CTAs per SM, one piece of global scratch each
+constexpr uint32_t MED_DISTINCT = 1536;      // distinct locations of a query on the medium path
 constexpr int SK_NW = 2;  // windows sketched together
 
 struct Cand {
@@ -689,7 +688,7 @@ __device__ __forceinline__ int query_score(const ClassifyDb& db, const ClassifyQ
 
 // Whole query on one warp with the bucket list in working memory.
 template <int R, int KC, class LocT, class CntT>
-__device__ __forceinline__ int process_query(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+__device__ __noinline__ int process_query(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
                                              const Scratch<CntT>& S, Counters& ctr) {
     uint32_t n_list = 0, sws = 0, n_feat = 0, n_sect = 0;
     int r = query_lookup<R, KC, LB_DEFAULT>(db, Q, q, S, S.list, n_list, sws, n_feat, n_sect);
@@ -1287,71 +1286,6 @@ __device__ __forceinline__ bool next_chunk_query(ChunkScan& it, const uint4* __r
     return true;
 }
 
-// One medium-path query (chunk index i): bucket list to working memory,
-// hash-histogram scoring; a query that does not fit is queued for the
-// large path.
-template <int GB, class KeyT, class LocT>
-__device__ __forceinline__ void medium_query(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q0,
-                                             uint32_t list_cap, const uint64_t* __restrict__ glist,
-                                             const Scratch<uint16_t, KeyT>& S, uint32_t i, const uint4& mt,
-                                             uint32_t* __restrict__ ovf_list, uint32_t* __restrict__ ovf_n,
-                                             Counters& ctr, unsigned long long& n_medium) {
-    const uint32_t lane = lane_id();
-    const uint64_t* src = glist + (uint64_t)i * list_cap;
-    for (uint32_t j = lane; j < mt.x; j += 32) S.list[j] = __ldg(src + j);
-    __syncwarp();
-    const uint32_t q = q0 + i;
-    if (query_score<GB, LocT>(db, Q, q, S, mt.x, meta_sws(mt), ctr) == Q_ESCALATE) {
-        if (lane == 0) ovf_list[atomicAdd(ovf_n, 1u)] = q;
-    } else {
-        ctr.features += meta_feat(mt);
-        ctr.found += mt.x;
-        ctr.sectors += mt.w;
-        ++ctr.queries;
-        ++n_medium;
-    }
-    __syncwarp();
-}
-
-// Medium path: the queries queued by the hash path's score kernel or the
-// sort path's largest size class, one warp each (work queue), KM_SLOTS
-// histogram slots per warp in shared memory, the bucket list taken over
-// from the lookup.  Queries that do not fit here either go to the large
-// path.
-template <int GB, class KeyT, class LocT>
-__global__ void __launch_bounds__(MED_WARPS * 32) k_classify_medium(ClassifyDb db, ClassifyQuery Q, uint32_t q0,
-                                                                   uint32_t list_cap,
-                                                                   const uint64_t* __restrict__ glist,
-                                                                   const uint4* __restrict__ meta,
-                                                                   const uint32_t* __restrict__ mid_list,
-                                                                   const uint32_t* __restrict__ mid_n,
-                                                                   uint32_t* __restrict__ mid_work,
-                                                                   uint32_t* __restrict__ ovf_list,
-                                                                   uint32_t* __restrict__ ovf_n) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t w = threadIdx.x >> 5;
-    const uint32_t lane = lane_id();
-    const size_t per_warp = scratch_bytes<uint16_t, KeyT>(KM_SLOTS, list_cap, 0, 0);
-    const Scratch<uint16_t, KeyT> S = carve<uint16_t, KeyT>(smem + w * per_warp, KM_SLOTS, list_cap, 0, 0, WIN_A);
-    Counters ctr;
-    unsigned long long n_medium = 0;
-    // a kernel launched after this one with programmatic stream
-    // serialization (a sort-path class, which shares no data with this one)
-    // may start while this one's few long queries finish
-    asm volatile("griddepcontrol.launch_dependents;");
-    const uint32_t n = *mid_n;
-    for (;;) {
-        uint32_t k = 0;
-        if (lane == 0) k = atomicAdd(mid_work, 1u);
-        k = __shfl_sync(FULL_MASK, k, 0);
-        if (k >= n) break;
-        const uint32_t i = mid_list[k];
-        medium_query<GB, KeyT, LocT>(db, Q, q0, list_cap, glist, S, i, meta[i], ovf_list, ovf_n, ctr, n_medium);
-    }
-    flush_counters(Q, ctr, KC_MEDIUM);
-    if (Q.counters && lane == 0 && n_medium) atomicAdd(Q.counters + 6, n_medium);
-}
-
 // ------------------------------------------------------------------
 // Sort path: query steps 5-8 of Section 5.2 for a query of at most 32*E
 // gathered locations, on one warp.  The paper compacts the gathered
@@ -1621,45 +1555,18 @@ __device__ __noinline__ void sort_to(LocT* dst, const LocT* src, uint32_t n) {
     }
 }
 
-// Steps 5-8 of a query from its n locations, sorted in loc: runs, scores,
+// Steps 6-8 of a query from its D distinct locations, ascending in loc, with
+// rs[j] = number of gathered locations below loc[j] (D + 1 entries): scores,
 // top m, label.  Locations may have been dropped with threshold T (see
 // above).  Returns 0 with the outputs written, or, if T turns out too high,
-// the threshold to use instead.
-// rs and score: working memory of n + 1 and n entries.
-template <class LocT>
-__device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q, LocT* loc,
-                                                 uint16_t* rs, uint16_t* score, uint32_t sws, uint32_t n, uint32_t T,
-                                                 uint32_t& distinct) {
+// the threshold to use instead.  score: working memory of D entries.
+template <class LocT, class IdxT>
+__device__ __forceinline__ uint32_t score_runs(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+                                               const LocT* loc, const IdxT* rs, IdxT* score, uint32_t sws, uint32_t D,
+                                               uint32_t T) {
     const uint32_t lane = lane_id();
-    const uint32_t lt = lanemask_lt();
     const uint32_t jb = sizeof(LocT) == 8 ? 32u : db.jbits;
     const uint32_t jmask = sizeof(LocT) == 8 ? 0xFFFFFFFFu : (1u << jb) - 1u;
-    // Runs of equal locations (the window count statistic of Section 5.6):
-    // run j has location loc[j] and covers sorted indices [rs[j], rs[j+1]).
-    // Written over the sorted locations: a run's index is at most its first
-    // element's, and a round's elements are read before its runs are written.
-    uint32_t D = 0;
-    LocT carry = 0;  // the element before the round's first
-    for (uint32_t base = 0; base < n; base += 32) {
-        const uint32_t i = base + lane;
-        const LocT x = i < n ? loc[i] : (LocT)0;
-        LocT prev = __shfl_up_sync(FULL_MASK, x, 1);
-        if (lane == 0) prev = carry;
-        carry = __shfl_sync(FULL_MASK, x, 31);
-        const bool start = i < n && (i == 0 || x != prev);
-        const uint32_t b = __ballot_sync(FULL_MASK, start);
-        if (start) {
-            const uint32_t pos = D + __popc(b & lt);
-            loc[pos] = x;
-            rs[pos] = (uint16_t)i;
-        }
-        D += __popc(b);
-        __syncwarp();
-    }
-    if (lane == 0) rs[D] = (uint16_t)n;
-    __syncwarp();
-    distinct = D;
-
     // Sliding-window scores (Section 5.6): the score of run j is the number
     // of sorted locations in [loc[j], hi], hi = loc[j] + sws - 1 cut at the
     // last window id of the target.  Runs have distinct locations, so at most
@@ -1682,7 +1589,7 @@ __device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const Cla
             if (adv < 4) break;
         }
         const uint32_t sc = (uint32_t)rs[e] - (uint32_t)rs[j];
-        score[j] = (uint16_t)sc;
+        score[j] = (IdxT)sc;
         const Cand c = Cand{sc, (uint32_t)(x >> jb), win, 0};
         if (better(c, best)) best = c;
     }
@@ -1759,6 +1666,42 @@ __device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const Cla
     }
     write_result(Q, q, label, hits, top, mine);
     return 0;
+}
+
+// Steps 5-8 of a query from its n locations, sorted in loc: runs of equal
+// locations (the window count statistic of Section 5.6), then score_runs.
+// Run j has location loc[j] and covers sorted indices [rs[j], rs[j+1]); the
+// runs are written over the sorted locations: a run's index is at most its
+// first element's, and a round's elements are read before its runs are
+// written.  rs and score: working memory of n + 1 and n entries.
+template <class LocT>
+__device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q, LocT* loc,
+                                                 uint16_t* rs, uint16_t* score, uint32_t sws, uint32_t n, uint32_t T,
+                                                 uint32_t& distinct) {
+    const uint32_t lane = lane_id();
+    const uint32_t lt = lanemask_lt();
+    uint32_t D = 0;
+    LocT carry = 0;  // the element before the round's first
+    for (uint32_t base = 0; base < n; base += 32) {
+        const uint32_t i = base + lane;
+        const LocT x = i < n ? loc[i] : (LocT)0;
+        LocT prev = __shfl_up_sync(FULL_MASK, x, 1);
+        if (lane == 0) prev = carry;
+        carry = __shfl_sync(FULL_MASK, x, 31);
+        const bool start = i < n && (i == 0 || x != prev);
+        const uint32_t b = __ballot_sync(FULL_MASK, start);
+        if (start) {
+            const uint32_t pos = D + __popc(b & lt);
+            loc[pos] = x;
+            rs[pos] = (uint16_t)i;
+        }
+        D += __popc(b);
+        __syncwarp();
+    }
+    if (lane == 0) rs[D] = (uint16_t)n;
+    __syncwarp();
+    distinct = D;
+    return score_runs<LocT, uint16_t>(db, Q, q, loc, rs, score, sws, D, T);
 }
 
 // One query of H <= 32*E locations, gathered in M.raw.  Returns false if its
@@ -1901,37 +1844,377 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Large path: queries queued by the shared-memory path, one warp each, with
-// working memory in global scratch.
+// ------------------------------------------------------------------
+// Queries beyond the sort path's size classes: one CTA per query.  All its
+// threads gather, count by block and drop locations as in query_sort, with
+// the two passes over the locations both reading them from global memory
+// (there may be any number); one warp then sorts and scores the survivors.
+// More than BLK_DISTINCT distinct survivors (which takes hundreds of equally
+// good targets) are left to the histogram code of one warp.
+//
+// One warp per query with a histogram took 0.6 ms for the slowest of a
+// launch of 2^20 pairs, whatever the others did (large database, 2 launches
+// 1.24 ms, here 0.71), and 5,000 reads of 1 to 6 kbp took 9.05 ms on
+// global-memory histograms, here 0.82.
+constexpr int BLK_THREADS = 256;
+constexpr int BLK_WARPS = BLK_THREADS / 32;
+constexpr uint32_t BLK_LIST = MC_MAX_QUERY_WINDOWS * MAX_S;  // buckets of one query
+constexpr uint32_t BLK_CNT = 4096;                           // block counters
+constexpr uint32_t BLK_HASH = 4096;                          // slots of the distinct survivors,
+constexpr uint32_t BLK_DISTINCT = 2048;                      // of which as many are used (what a warp sorts)
+constexpr int BLK_STEP = 8;                                  // consecutive locations per thread and step
+
+template <class LocT>
+struct BlockMem {
+    uint64_t list[BLK_LIST];      // found buckets, offset << 16 | size
+    uint32_t pre[BLK_LIST + 4];   // exclusive prefix of their sizes
+    uint32_t cnt[BLK_CNT];
+    LocT key[BLK_HASH];           // distinct surviving locations, hashed,
+    uint32_t times[BLK_HASH];     // and how often each was gathered
+    LocT loc[BLK_DISTINCT + 4];   // the same sorted
+    uint32_t rs[BLK_DISTINCT + 4];
+    union {
+        uint32_t score[BLK_DISTINCT + 4];
+        uint32_t feat[BLK_LIST];  // (before the scores) the windows' features
+    };
+    uint64_t waddr[MC_MAX_QUERY_WINDOWS];  // windows: address of the first base,
+    uint32_t wnk[MC_MAX_QUERY_WINDOWS];    // k-mers, features
+    uint32_t wcnt[MC_MAX_QUERY_WINDOWS];
+    uint32_t cand[BLK_WARPS][32];
+    uint32_t part[BLK_WARPS];     // block-wide scan and maximum
+    uint32_t n_list, sect, n, T, n_win, sws, n_feat, work;
+    int status;
+};
+
+// f(location) for every location of the query's n_list buckets (H in all).
+template <class LocT, class F>
+__device__ __forceinline__ void block_for_each(const ClassifyDb& db, const BlockMem<LocT>& B, uint32_t n_list,
+                                               uint32_t H, F f) {
+    const LocT* __restrict__ locs = static_cast<const LocT*>(db.locs);
+    for (uint32_t x0 = threadIdx.x * BLK_STEP; x0 < H; x0 += BLK_THREADS * BLK_STEP) {
+        uint32_t lo = 0, hi = n_list;  // last bucket with pre <= x0
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (B.pre[mid] <= x0) lo = mid; else hi = mid;
+        }
+        LocT v[BLK_STEP];
+#pragma unroll
+        for (int u = 0; u < BLK_STEP; ++u) {
+            const uint32_t x = x0 + u;
+            v[u] = 0;
+            if (x < H) {
+                while (B.pre[lo + 1] <= x) ++lo;
+                v[u] = __ldcg(locs + (B.list[lo] >> 16) + (x - B.pre[lo]));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < BLK_STEP; ++u)
+            if (x0 + u < H) f(v[u]);
+    }
+}
+
+// Steps 5-8 of the query whose n_list buckets are in B.list, by the whole
+// CTA (called between barriers; ends with one).  The surviving locations are
+// made distinct by a hash table before they are sorted: repeats and long
+// queries gather the same ones many times.  False: more than d_max of them.
+template <class LocT>
+__device__ __forceinline__ bool block_score(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+                                            BlockMem<LocT>& B, uint32_t n_list, uint32_t sws, uint32_t d_max,
+                                            uint32_t& H_out, uint32_t& distinct) {
+    constexpr uint32_t MASK = BLK_CNT - 1;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
+    BlockSlot<LocT> bs;
+    bs.jb = sizeof(LocT) == 8 ? 32u : db.jbits;
+    bs.jmask = sizeof(LocT) == 8 ? 0xFFFFFFFFu : (1u << bs.jb) - 1u;
+    bs.b = sws > 1 ? 32u - (uint32_t)__clz(sws - 1) : 0u;
+    // exclusive prefix of the bucket sizes: eight buckets per thread
+    constexpr uint32_t PER = BLK_LIST / BLK_THREADS;
+    uint32_t sum = 0;
+    for (uint32_t i = tid * PER; i < min((tid + 1) * PER, n_list); ++i) sum += (uint32_t)B.list[i] & 0xFFFFu;
+    uint32_t inc = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t x = __shfl_up_sync(FULL_MASK, inc, d);
+        if ((int)lane >= d) inc += x;
+    }
+    if (lane == 31) B.part[w] = inc;
+    for (uint32_t i = tid; i < BLK_CNT; i += BLK_THREADS) B.cnt[i] = 0;
+    __syncthreads();
+    uint32_t H = 0, at = inc - sum;
+    for (uint32_t i = 0; i < BLK_WARPS; ++i) {
+        if (i < w) at += B.part[i];
+        H += B.part[i];
+    }
+    for (uint32_t i = tid * PER; i < min((tid + 1) * PER, n_list); ++i) {
+        B.pre[i] = at;
+        at += (uint32_t)B.list[i] & 0xFFFFu;
+    }
+    if (tid == 0) B.pre[n_list] = H;
+    H_out = H;
+    __syncthreads();
+    uint32_t T = Q.counters ? 1u : 0u;
+    if (T == 0) {
+        block_for_each(db, B, n_list, H, [&](LocT x) { atomicAdd(&B.cnt[bs(x, MASK)], 1u); });
+        __syncthreads();
+        uint32_t most = 0;
+        for (uint32_t s = tid; s < BLK_CNT; s += BLK_THREADS)
+            if (B.cnt[s]) most = max(most, B.cnt[s] + max(B.cnt[(s - 1) & MASK], B.cnt[(s + 1) & MASK]));
+        most = __reduce_max_sync(FULL_MASK, most);
+        if (lane == 0) B.part[w] = most;
+        __syncthreads();
+        for (uint32_t i = 0; i < BLK_WARPS; ++i) most = max(most, B.part[i]);
+        const uint64_t close = ((uint64_t)(100 - Q.band) * most + 99) / 100;
+        T = max(Q.cands ? most / 4 : (uint32_t)(close - close / 8), 1u);
+    }
+    constexpr LocT EMPTY = KeyCodec<LocT>::empty();
+    for (;;) {
+        for (uint32_t i = tid; i < BLK_HASH; i += BLK_THREADS) {
+            B.key[i] = EMPTY;
+            B.times[i] = 0;
+        }
+        if (tid == 0) B.n = 0;
+        __syncthreads();
+        block_for_each(db, B, n_list, H, [&](LocT x) {
+            if (T > 1) {
+                const uint32_t s = bs(x, MASK);
+                if (B.cnt[s] + max(B.cnt[(s - 1) & MASK], B.cnt[(s + 1) & MASK]) < T) return;
+            }
+            // (the threads together pass the limit by at most one each, so
+            // the table never fills)
+            if (*(volatile uint32_t*)&B.n > d_max) return;
+            int fresh = -1;
+            hist_insert(B.key, B.times, BLK_HASH - 1, x, fresh);
+            if (fresh >= 0) atomicAdd(&B.n, 1u);
+        });
+        __syncthreads();
+        const uint32_t D = B.n;
+        __syncthreads();
+        if (D > d_max) return false;
+        if (tid == 0) B.n = 0;
+        __syncthreads();
+        for (uint32_t i = tid; i < BLK_HASH; i += BLK_THREADS)
+            if (B.key[i] != EMPTY) B.loc[atomicAdd(&B.n, 1u)] = B.key[i];
+        __syncthreads();
+        if (w == 0) {
+            const LocT* from = B.loc;  // sorted in place
+            if (D <= 32) sort_to<1>(B.loc, from, D);
+            else if (D <= 64) sort_to<2>(B.loc, from, D);
+            else if (D <= 256) sort_to<8>(B.loc, from, D);
+            else if (D <= 512) sort_to<16>(B.loc, from, D);
+            else if (D <= 1024) sort_to<32>(B.loc, from, D);
+            else sort_to<64>(B.loc, from, D);
+            __syncwarp();
+            uint32_t before = 0;
+            for (uint32_t j0 = 0; j0 < D; j0 += 32) {
+                const uint32_t j = j0 + lane;
+                uint32_t c = j < D ? hist_count(B.key, B.times, BLK_HASH - 1, B.loc[j]) : 0u;
+                uint32_t pre = c;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t x = __shfl_up_sync(FULL_MASK, pre, d);
+                    if ((int)lane >= d) pre += x;
+                }
+                if (j < D) B.rs[j] = before + pre - c;
+                before += __shfl_sync(FULL_MASK, pre, 31);
+            }
+            if (lane == 0) B.rs[D] = before;
+            __syncwarp();
+            const uint32_t t2 = score_runs<LocT, uint32_t>(db, Q, q, B.loc, B.rs, B.score, sws, D, T);
+            if (lane == 0) B.T = t2;
+        }
+        __syncthreads();
+        T = B.T;
+        distinct = D;
+        if (T == 0) return true;
+    }
+}
+
+// Medium path: the queries queued by the hash path's score kernel or the
+// sort path's classes, one CTA each (work queue), the bucket list taken
+// over from the lookup; queries of more than MED_DISTINCT distinct locations
+// go to the large path.
+template <class LocT>
+__global__ void __launch_bounds__(BLK_THREADS, 2) k_classify_medium(ClassifyDb db, ClassifyQuery Q, uint32_t q0,
+                                                                   uint32_t list_cap,
+                                                                   const uint64_t* __restrict__ glist,
+                                                                   const uint4* __restrict__ meta,
+                                                                   const uint32_t* __restrict__ mid_list,
+                                                                   const uint32_t* __restrict__ mid_n,
+                                                                   uint32_t* __restrict__ mid_work,
+                                                                   uint32_t* __restrict__ ovf_list,
+                                                                   uint32_t* __restrict__ ovf_n) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    BlockMem<LocT>& B = *reinterpret_cast<BlockMem<LocT>*>(smem);
+    // a kernel launched after this one with programmatic stream
+    // serialization (a sort-path class, which shares no data with this one)
+    // may start while this one's few long queries finish
+    asm volatile("griddepcontrol.launch_dependents;");
+    const uint32_t n = *mid_n;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) B.work = atomicAdd(mid_work, 1u);
+        __syncthreads();
+        const uint32_t k = B.work;
+        if (k >= n) break;
+        const uint32_t i = mid_list[k];
+        const uint4 mt = meta[i];
+        const uint64_t* src = glist + (uint64_t)i * list_cap;
+        for (uint32_t j = threadIdx.x; j < mt.x; j += BLK_THREADS) B.list[j] = __ldg(src + j);
+        __syncthreads();
+        uint32_t H = 0;
+        uint32_t distinct = 0;
+        const bool done = block_score<LocT>(db, Q, q0 + i, B, mt.x, meta_sws(mt), MED_DISTINCT, H, distinct);
+        if (!done && threadIdx.x == 0) ovf_list[atomicAdd(ovf_n, 1u)] = q0 + i;
+        if (Q.counters && done && threadIdx.x < 32) {
+            Counters ctr;
+            ctr.locations = H;
+            ctr.distinct = distinct;
+            ctr.features = meta_feat(mt);
+            ctr.found = mt.x;
+            ctr.sectors = mt.w;
+            ctr.queries = 1;
+            flush_counters(Q, ctr, KC_MEDIUM);
+            if (threadIdx.x == 0) atomicAdd(Q.counters + 6, 1ull);
+        }
+    }
+}
+
+// Windows, sketches and table probes of a query of the large path by the
+// whole CTA: fills B.list, B.n_list, B.sws, B.n_feat, B.sect; B.status is
+// Q_DONE, or else the query is beyond the large path's limits.  Ends with a
+// barrier.
 template <int R, int KC, class LocT>
-__global__ void __launch_bounds__(CLS_WARPS * 32, 4) k_classify_large(ClassifyDb db, ClassifyQuery Q,
+__device__ __forceinline__ void block_lookup(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+                                             BlockMem<LocT>& B) {
+    const SketchParams& p = db.sp;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
+    const uint32_t k = KC ? (uint32_t)KC : p.k;
+    if (w == 0) {  // lane i holds mate i
+        const QueryIn in = query_in(Q, q);
+        const bool mates_ok = in.m1 >= in.m0 && in.m1 - in.m0 <= MAX_MATES;
+        const uint32_t nm = mates_ok ? in.m1 - in.m0 : 0u;
+        const uint64_t o = mates_ok && lane <= nm ? in.offs[in.m0 + lane] : 0;
+        const uint64_t o_next = __shfl_down_sync(FULL_MASK, o, 1);
+        const uint64_t L = (lane < nm && o_next > o) ? o_next - o : 0;
+        const uint64_t nw = num_windows(L, k, p.stride);
+        const uint64_t span = warp_sum_u64(L), n_win = warp_sum_u64(nw);
+        const bool fits = mates_ok && n_win <= MC_MAX_QUERY_WINDOWS && span <= BUF_B;
+        if (fits) {
+            uint32_t off = (uint32_t)L, wat = (uint32_t)nw;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t x = __shfl_up_sync(FULL_MASK, off, d), y = __shfl_up_sync(FULL_MASK, wat, d);
+                if ((int)lane >= d) {
+                    off += x;
+                    wat += y;
+                }
+            }
+            off -= (uint32_t)L;
+            wat -= (uint32_t)nw;
+            const uint64_t base = (uint64_t)(uintptr_t)in.seq + __shfl_sync(FULL_MASK, o, 0) + off;
+            for (uint32_t j = 0; j < (uint32_t)nw; ++j) {
+                const uint32_t ws = j * p.stride;
+                B.waddr[wat + j] = base + ws;
+                B.wnk[wat + j] = min(p.w, (uint32_t)L - ws) - k + 1;
+            }
+        }
+        if (lane == 0) {
+            const uint64_t sp = nm <= 1 ? span : (span > Q.max_insert ? span : (uint64_t)Q.max_insert);
+            B.status = fits ? Q_DONE : Q_TOO_LARGE;
+            B.n_win = fits ? (uint32_t)n_win : 0u;
+            B.sws = fits && sp >= k ? (uint32_t)((sp - k + p.stride - 1) / p.stride + 1) : 0u;
+            B.n_list = B.n_feat = B.sect = 0;
+        }
+    }
+    __syncthreads();
+    const uint32_t n_win = B.n_win;
+    for (uint32_t j = w; j < n_win; j += BLK_WARPS) {
+        const uint8_t* const sq[1] = {reinterpret_cast<const uint8_t*>(B.waddr[j])};
+        const uint64_t Ls[1] = {B.wnk[j] + k - 1}, wss[1] = {0};
+        const bool on[1] = {true};
+        uint32_t f[1], c[1];
+        warp_sketch_multi<R, 1, KC>(sq, Ls, wss, on, p, B.cand[w], f, c);
+        if (lane < c[0]) B.feat[j * p.s + lane] = f[0];
+        if (lane == 0) {
+            B.wcnt[j] = c[0];
+            atomicAdd(&B.n_feat, c[0]);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    const TableProbe tp(db.fmt);
+    const uint32_t lsz = sizeof(LocT);
+    for (uint32_t x = tid; x < n_win * p.s; x += BLK_THREADS) {
+        const uint32_t j = x / p.s;
+        if (x - j * p.s >= B.wcnt[j]) continue;
+        const uint32_t h = hash_h2(B.feat[x]);
+        const uint64_t home = tp.home(h);
+        const uint64_t* t = db.table + home;
+        for (uint32_t d = 0; d <= db.max_probe; ++d) {
+            const uint64_t e = __ldcg(t + d);
+            const uint32_t what = tp.step(e, d, h);
+            if (what == 2) continue;
+            if (what == 1) {
+                const uint64_t bk = tp.bucket(e);
+                B.list[atomicAdd(&B.n_list, 1u)] = bk;
+                const uint64_t lo = (bk >> 16) * lsz, hi = lo + (bk & 0xFFFFu) * lsz - 1;
+                atomicAdd(&B.sect, (uint32_t)((hi >> 5) - (lo >> 5) + 1));
+            }
+            break;
+        }
+    }
+    __syncthreads();
+}
+
+// Large path: queries with too many windows or bases for the lookup kernels
+// and those that the medium path does not hold (the queue ovf_list), or, in a
+// launch of few queries (ovf_list null), all of them; one CTA each; what does not
+// fit the CTA's memory is processed by one warp with working memory in
+// global scratch (one piece per CTA).
+template <int R, int KC, class LocT>
+__global__ void __launch_bounds__(BLK_THREADS, 2) k_classify_large(ClassifyDb db, ClassifyQuery Q,
                                                                    const uint32_t* __restrict__ ovf_list,
                                                                    const uint32_t* __restrict__ ovf_n,
                                                                    uint32_t* __restrict__ work,
                                                                    unsigned char* __restrict__ scratch,
-                                                                   size_t per_warp) {
-    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const Scratch<uint32_t> S =
-        carve<uint32_t>(scratch + gw * per_warp, KB_SLOTS, LIST_B, LIST_B, BUF_B, MC_MAX_QUERY_WINDOWS);
-    Counters ctr;
-    const uint32_t n = *ovf_n;
-    unsigned long long n_large = 0;
-    for (;;) {
-        uint32_t i = 0;
-        if (lane_id() == 0) i = atomicAdd(work, 1u);
-        i = __shfl_sync(FULL_MASK, i, 0);
+                                                                   size_t per_cta) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    BlockMem<LocT>& B = *reinterpret_cast<BlockMem<LocT>*>(smem);
+    const uint32_t n = ovf_list ? *ovf_n : total_queries(Q);
+    for (uint32_t turn = 0;; ++turn) {
+        __syncthreads();
+        if (threadIdx.x == 0) B.work = ovf_list ? atomicAdd(work, 1u) : turn * gridDim.x + blockIdx.x;
+        __syncthreads();
+        const uint32_t i = B.work;
         if (i >= n) break;
-        const uint32_t q = ovf_list[i];
-        ++n_large;
-        int r = process_query<R, KC, LocT>(db, Q, q, S, ctr);
-        if (r != Q_DONE) {
-            write_unclassified(Q, q);
-            if (lane_id() == 0) atomicMax(Q.status, DEV_ERR_CAPACITY);
+        const uint32_t q = ovf_list ? ovf_list[i] : i;
+        block_lookup<R, KC, LocT>(db, Q, q, B);
+        bool done = false;
+        uint32_t H = 0, distinct = 0;
+        if (B.status == Q_DONE) done = block_score<LocT>(db, Q, q, B, B.n_list, B.sws, BLK_DISTINCT, H, distinct);
+        if (threadIdx.x < 32) {
+            Counters ctr;
+            if (done) {
+                ctr.features = B.n_feat;
+                ctr.locations = H;
+                ctr.distinct = distinct;
+                ctr.found = B.n_list;
+                ctr.sectors = B.sect;
+                ctr.queries = 1;
+            } else {
+                const Scratch<uint32_t> S = carve<uint32_t>(scratch + blockIdx.x * per_cta, KB_SLOTS, LIST_B, LIST_B,
+                                                            BUF_B, MC_MAX_QUERY_WINDOWS);
+                if (process_query<R, KC, LocT>(db, Q, q, S, ctr) != Q_DONE) {
+                    write_unclassified(Q, q);
+                    if (threadIdx.x == 0) atomicMax(Q.status, DEV_ERR_CAPACITY);
+                }
+            }
+            if (Q.counters) {
+                flush_counters(Q, ctr, KC_LARGE);
+                if (threadIdx.x == 0) atomicAdd(Q.counters + 3, 1ull);
+            }
         }
-        __syncwarp();
     }
-    flush_counters(Q, ctr, KC_LARGE);
-    if (Q.counters && lane_id() == 0 && n_large) atomicAdd(Q.counters + 3, n_large);
 }
 
 
@@ -2012,9 +2295,7 @@ ScoreKernel pick_score(uint32_t ka, uint32_t gb, KeyMode km) {
 }
 
 MediumKernel pick_medium(KeyMode km) {
-    if (km == KeyMode::compact) return k_classify_medium<GB_DEFAULT, uint32_t, uint32_t>;
-    if (km == KeyMode::wide32) return k_classify_medium<GB_DEFAULT, uint64_t, uint32_t>;
-    return k_classify_medium<GB_DEFAULT, uint64_t, uint64_t>;
+    return km == KeyMode::wide64 ? k_classify_medium<uint64_t> : k_classify_medium<uint32_t>;
 }
 
 template <class LocT>
@@ -2057,10 +2338,31 @@ struct Geometry {
     bool sort;           // score by the sort path (else the hash path)
     int n_sort;          // sort classes in use
     uint32_t list_cap;
-    size_t smem_l, smem_s, smem_m, per_warp_b, smem_t[N_SORT_CLASSES];
+    size_t smem_l, smem_s, smem_m, smem_b, per_warp_b, smem_t[N_SORT_CLASSES];
     uint32_t threads_l, threads_s, grid_l, grid_s, grid_m, blocks_b, grid_t[N_SORT_CLASSES];
     uint32_t group_shift;  // log2 of the queries a sort-path warp takes at a time
 };
+
+// Resident CTAs per SM of a kernel, remembered per thread: the query takes
+// several microseconds, and a call that classifies a handful of queries makes
+// five of them.  A function of the kernel, the launch shape and the device.
+cudaError_t resident_ctas(const void* kernel, uint32_t threads, size_t smem, int dev, int* out) {
+    struct Known {
+        const void* kernel;
+        size_t smem;
+        uint32_t threads;
+        int dev, ctas;
+    };
+    thread_local std::vector<Known> known;
+    for (const Known& k : known)
+        if (k.kernel == kernel && k.smem == smem && k.threads == threads && k.dev == dev) {
+            *out = k.ctas;
+            return cudaSuccess;
+        }
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, (int)threads, smem);
+    if (e == cudaSuccess) known.push_back(Known{kernel, smem, threads, dev, *out});
+    return e;
+}
 
 cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratch& sc, Geometry* g) {
     cudaError_t e;
@@ -2076,14 +2378,14 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->ks = pick_score(t.hist_slots, t.gather_batch, km);
     g->kb = pick_large(db);
     g->km = pick_medium(km);
-    g->smem_m = MED_WARPS * (compact ? scratch_bytes<uint16_t, uint32_t>(KM_SLOTS, g->list_cap, 0, 0)
-                                     : scratch_bytes<uint16_t, uint64_t>(KM_SLOTS, g->list_cap, 0, 0));
+    const size_t blk = db.jbits ? sizeof(BlockMem<uint32_t>) : sizeof(BlockMem<uint64_t>);
+    g->smem_b = blk;
+    g->smem_m = blk;
     if ((e = cudaFuncSetAttribute(g->km, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_m)) != cudaSuccess)
         return e;
-    int occ_m = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_m, g->km, MED_WARPS * 32, g->smem_m)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(g->kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_b)) != cudaSuccess)
         return e;
-    g->grid_m = (uint32_t)sms * (uint32_t)std::max(occ_m, 1);
+    g->grid_m = std::min<uint32_t>((uint32_t)sms * 2, std::max<uint32_t>(sc.chunk, 1));
     g->threads_l = t.lookup_warps * 32;
     g->threads_s = t.score_warps * 32;
     g->smem_l = t.lookup_warps * (g->kll ? sizeof(LookupLanesMem) : lookup_warp_bytes(g->list_cap));
@@ -2094,9 +2396,9 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     if ((e = cudaFuncSetAttribute(g->ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_s)) != cudaSuccess)
         return e;
     int occ_l = 1, occ_s = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_l, kl_any, g->threads_l, g->smem_l)) != cudaSuccess)
+    if ((e = resident_ctas(kl_any, g->threads_l, g->smem_l, dev, &occ_l)) != cudaSuccess)
         return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, g->ks, g->threads_s, g->smem_s)) != cudaSuccess)
+    if ((e = resident_ctas((const void*)g->ks, g->threads_s, g->smem_s, dev, &occ_s)) != cudaSuccess)
         return e;
     occ_l = std::max(occ_l, 1);
     occ_s = std::max(occ_s, 1);
@@ -2112,7 +2414,7 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     }
     g->grid_s = (uint32_t)std::min<uint64_t>((c + t.score_warps - 1) / t.score_warps, (uint64_t)sms * occ_s);
     g->per_warp_b = scratch_bytes<uint32_t>(KB_SLOTS, LIST_B, LIST_B, BUF_B);
-    g->blocks_b = std::max<uint32_t>(1, sc.large_warps / CLS_WARPS);
+    g->blocks_b = std::max<uint32_t>(1, std::min(sc.large_warps, sc.n_q_cap));  // one piece of global scratch each
     // sort path: locations sorted as they are stored (not with wide keys of 32-bit ones)
     g->sort = km != KeyMode::wide32 && t.score_mode != SCORE_HASH;
     g->n_sort = 0;
@@ -2141,7 +2443,7 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
                 cudaSuccess)
                 return e;
             int occ_t = 1;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_t, kts[c2], SORT_WARPS * 32, g->smem_t[c2])) !=
+            if ((e = resident_ctas((const void*)kts[c2], SORT_WARPS * 32, g->smem_t[c2], dev, &occ_t)) !=
                 cudaSuccess)
                 return e;
             g->grid_t[c2] = (uint32_t)std::min<uint64_t>((c + SORT_WARPS - 1) / SORT_WARPS,
@@ -2199,8 +2501,27 @@ cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const Classif
                           uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
     MC_LAUNCH("classify_medium", s,
-              g.km<<<g.grid_m, MED_WARPS * 32, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid, qc + 2,
+              g.km<<<g.grid_m, BLK_THREADS, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid, qc + 2,
                                                              qc + 3, sc.ovf, qc));
+    return cudaGetLastError();
+}
+
+// A launch of few queries: all of them straight to the large path's kernel.
+// One launch instead of the six kernels and three memsets of a launch set,
+// whose latency is what such a call takes: 16 pairs 25 us on the device
+// against 65.  One wave of CTAs (two per SM) holds 304 queries; 2,000 take
+// 115 us this way and 61 the other (reads of 100), so the line lies between.
+constexpr uint32_t DIRECT_MAX_QUERIES = 512;
+
+cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc, cudaStream_t s) {
+    const LargeKernel kb = pick_large(db);
+    const size_t smem = db.jbits ? sizeof(BlockMem<uint32_t>) : sizeof(BlockMem<uint64_t>);
+    cudaError_t e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const uint32_t grid = std::max<uint32_t>(1, std::min(sc.large_warps, Q.n_q));
+    MC_LAUNCH("classify_large", s,
+              kb<<<grid, BLK_THREADS, smem, s>>>(db, Q, nullptr, nullptr, nullptr, sc.large,
+                                                scratch_bytes<uint32_t>(KB_SLOTS, LIST_B, LIST_B, BUF_B)));
     return cudaGetLastError();
 }
 
@@ -2270,7 +2591,7 @@ cudaError_t launch_large(const Geometry& g, const ClassifyDb& db, const Classify
                          cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
     MC_LAUNCH("classify_large", s,
-              g.kb<<<g.blocks_b, CLS_WARPS * 32, 0, s>>>(db, Q, sc.ovf, qc, qc + 1, sc.large, g.per_warp_b));
+              g.kb<<<g.blocks_b, BLK_THREADS, g.smem_b, s>>>(db, Q, sc.ovf, qc, qc + 1, sc.large, g.per_warp_b));
     return cudaGetLastError();
 }
 
@@ -2396,7 +2717,7 @@ uint32_t classify_default_large_warps() {
         cudaGetLastError();
         sms = NUM_SMS_HINT;
     }
-    return (uint32_t)std::max(CLS_WARPS, (sms * B_WARPS_PER_SM / CLS_WARPS) * CLS_WARPS);
+    return (uint32_t)(sms * B_WARPS_PER_SM);
 }
 
 size_t classify_scratch_bytes(uint32_t n_q_cap, uint32_t sketch_size, uint32_t large_warps) {
@@ -2425,6 +2746,11 @@ cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const
     if (n_kernels) *n_kernels = 0;
     if (Q.n_q == 0) return cudaSuccess;
     if (Q.n_q > sc.n_q_cap) return cudaErrorInvalidValue;
+    if (Q.n_q <= DIRECT_MAX_QUERIES && !Q.counters) {
+        if ((e = launch_direct(db, Q, sc, s)) != cudaSuccess) return e;
+        if (n_kernels) *n_kernels = 1;
+        return cudaSuccess;
+    }
     Geometry g;
     if ((e = geometry(db, t, sc, &g)) != cudaSuccess) return e;
     // only the queue counters must start at zero
@@ -2450,7 +2776,7 @@ cudaError_t classify_launch(const Mem& mem, const ClassifyDb& db, const Classify
     return classify_enqueue(db, Q, t, sc, s, nullptr);
 }
 
-// Number of large-path warps of the allocation-free launch.
+// Number of large-path CTAs of the allocation-free launch.
 constexpr uint32_t NOALLOC_LARGE_WARPS = 8;
 // The documented per-call maximum of the allocation-free entry point must
 // fit its fixed scratch array at the largest sketch size.

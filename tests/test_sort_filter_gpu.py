@@ -1,4 +1,4 @@
-"""The sort path's filter (locations whose target and window block are hit
+"""Classification's filter (locations whose target and window block are hit
 too rarely to matter are dropped before the sort) against the oracle: where
 the bound that guides it is tight and where it is not (tandem copies next to
 each other double it), with every survivor count from none to all, location
@@ -62,25 +62,37 @@ def _queries(rng, targets, unit):
         qs.append([unit[a:a + rng.choice([60, 128, 200])], unit[rng.randrange(600):][:rng.choice([30, 128, 250])]])
     qs += [[_rand(rng, 150), _rand(rng, 150)] for _ in range(60)]
     qs += [[targets[rng.randrange(9)][50:150], _rand(rng, 100), targets[20][300:400]] for _ in range(30)]
+    # invalid bases, lower case, empty and short mates, long reads, repeats, no mates
+    qs += [[x[:n] + "N" + x[n + 1:].lower() for x in q] for n, q in zip(range(40), qs)]
+    qs += [[], [""], ["ACGT"], ["", targets[0][:200]], ["N" * 200], ["A" * 200, "ACGT" * 60], [targets[0][:6000]]]
+    qs += [[targets[i][:n]] for i in range(9) for n in (900, 1030, 3000)] + [[t[:400] for t in targets[:9]]]
     return qs
 
 
-def _check(mc, db, odb, parent, taxon, qs, m, with_cands, **cp):
-    import torch
+def _reads(qs):
     mates = [x for q in qs for x in q]
-    reads = u8("".join(mates))
-    roffs = offsets([len(x) for x in mates])
     qoffs = np.zeros(len(qs) + 1, np.uint32)
     qoffs[1:] = np.cumsum([len(q) for q in qs])
-    cands = torch.zeros(len(qs) * m * 4, dtype=torch.int32, device="cuda") if with_cands else None
-    got = db.classify(dev(reads), dev(roffs), dev(qoffs), cands=cands, max_candidates=m, **cp)
-    mc.mc_classify_status(db.handle)
-    want = odb.classify(parent, taxon, reads, roffs, qoffs, max_candidates=m, with_cands=True, n_threads=8, **cp)
-    for g, o in zip(got, want[:3]):
-        bad = np.nonzero(host_u32(g) != o)[0]
-        assert len(bad) == 0, bad[:10]
-    if with_cands:
-        assert (host_u32(cands).reshape(len(qs), m, 4) == want[3]).all()
+    return u8("".join(mates)), offsets([len(x) for x in mates]), qoffs
+
+
+def _check(mc, db, odb, parent, taxon, qs, m, with_cands, sizes=(0, 1100, 33000), **cp):
+    """The queries as they are (few: one CTA per query) and repeated until
+    there are as many as the sort path and the lane-wide lookup start at."""
+    import torch
+    want = odb.classify(parent, taxon, *_reads(qs), max_candidates=m, with_cands=True, n_threads=8, **cp)
+    for size in sizes:
+        reps = max(1, -(-size // len(qs)))
+        reads, roffs, qoffs = _reads(qs * reps)
+        n = len(qoffs) - 1
+        cands = torch.zeros(n * m * 4, dtype=torch.int32, device="cuda") if with_cands else None
+        got = db.classify(dev(reads), dev(roffs), dev(qoffs), cands=cands, max_candidates=m, **cp)
+        mc.mc_classify_status(db.handle)
+        for g, o in zip(got, want[:3]):
+            bad = np.nonzero(host_u32(g) != np.tile(o, reps))[0]
+            assert len(bad) == 0, (size, bad[:10])
+        if with_cands:
+            assert (host_u32(cands).reshape(n, m, 4) == np.tile(want[3], (reps, 1, 1))).all()
 
 
 @pytest.fixture(scope="module")
@@ -120,8 +132,8 @@ def test_class_edges(mc, copies):
     try:
         qs = [[unit], [unit[:60]], [unit, unit[:100]], [_mutated(rng, unit, 0.03)]] * 9
         for with_cands in (False, True):
-            _check(mc, db, oracle.DB(seq, goffs, **P), parent, taxon, qs, 4, with_cands, hits_min=1, lca_band_pct=10,
-                   max_insert=0)
+            _check(mc, db, oracle.DB(seq, goffs, **P), parent, taxon, qs, 4, with_cands, sizes=(0, 1100), hits_min=1,
+                   lca_band_pct=10, max_insert=0)
     finally:
         db.free()
 
