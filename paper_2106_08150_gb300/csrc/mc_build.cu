@@ -43,9 +43,6 @@ inline uint32_t grid_for(uint64_t tiles, uint32_t per_sm = 8) {
 struct OpSum {
     __device__ __forceinline__ uint64_t operator()(uint64_t a, uint64_t b) const { return a + b; }
 };
-struct OpMaxU {
-    __device__ __forceinline__ uint64_t operator()(uint64_t a, uint64_t b) const { return a > b ? a : b; }
-};
 struct OpMaxI {
     __device__ __forceinline__ int64_t operator()(int64_t a, int64_t b) const { return a > b ? a : b; }
 };
@@ -826,35 +823,37 @@ __global__ void __launch_bounds__(BT) k_fin_count(const uint64_t* __restrict__ a
 
 // Writes the condensed outputs at the scanned positions: locations of kept
 // pairs (global window -> (target, window), 32-bit target << jbits | window
-// when jbits > 0, else 64-bit target << 32 | window), and per feature its h2 value,
-// the position of its first location and the index of its first pair.
+// when jbits > 0, else 64-bit target << 32 | window), and per feature its h2
+// value and the position of its first location.
 // The target of a global window gw is the last t with wbase[t] <= gw; a
 // block first tabulates that target for the first window of each of
 // FIN_BUCKETS equal window ranges, which narrows every search to the
-// targets that overlap gw's range (one or two for genome-sized targets).
-// With wb_smem, wbase (n_targets + 1 words) is copied to shared memory too,
-// so that the search and the window offset are shared-memory reads.
-__global__ void __launch_bounds__(BT) k_fin_emit(const uint64_t* __restrict__ a, uint64_t n, uint32_t cap,
-                                                 const uint64_t* __restrict__ tkept, const uint64_t* __restrict__ tkeys,
-                                                 uint64_t n_tiles, const uint32_t* __restrict__ wbase,
-                                                 uint32_t n_targets, uint32_t jbits, void* __restrict__ locs,
-                                                 uint32_t* __restrict__ khk, uint64_t* __restrict__ koff,
-                                                 uint64_t* __restrict__ kstart, unsigned long long* overflow,
-                                                 bool wb_smem) {
+// targets that overlap gw's range (a few for genome-sized targets).  WB:
+// wbase (n_targets + 1 words) is copied to shared memory too.
+// A thread's items are searched four at a time, one step of each per round,
+// so that their reads overlap, and a pair's predecessor comes from the lane
+// before it.  Bound by latency and issue (the pairs are read and the
+// locations written once, 28 GB on the large workload, 4 ms).
+template <bool WB>
+__global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__ a, uint64_t n, uint32_t cap,
+                                                    const uint64_t* __restrict__ tkept, const uint64_t* __restrict__ tkeys,
+                                                    uint64_t n_tiles, const uint32_t* __restrict__ wbase,
+                                                    uint32_t n_targets, uint32_t jbits, void* __restrict__ locs,
+                                                    uint32_t* __restrict__ khk, uint64_t* __restrict__ koff,
+                                                    unsigned long long* overflow) {
     extern __shared__ uint32_t fin_smem[];
     uint32_t* first_target = fin_smem;  // FIN_BUCKETS + 1 words
+    uint32_t* copy = fin_smem + FIN_BUCKETS + 1;
     __shared__ uint32_t wk[NWARP], wsx[NWARP];
     const int w = threadIdx.x >> 5;
     const uint32_t lane = lane_id();
     const uint32_t lt = lanemask_lt();
-    const uint32_t* wb = wbase;
-    if (wb_smem) {
-        uint32_t* copy = fin_smem + FIN_BUCKETS + 1;
+    if (WB) {
         for (uint32_t t = threadIdx.x; t <= n_targets; t += BT) copy[t] = wbase[t];
         __syncthreads();
-        wb = copy;
     }
-    const uint64_t n_win = wb[n_targets];
+    const auto wb = [&](uint32_t t) { return WB ? copy[t] : __ldg(wbase + t); };
+    const uint64_t n_win = wb(n_targets);
     uint32_t bshift = 0;
     while ((n_win >> bshift) >= FIN_BUCKETS) ++bshift;
     for (uint32_t b = threadIdx.x; b <= FIN_BUCKETS; b += BT) {
@@ -862,26 +861,41 @@ __global__ void __launch_bounds__(BT) k_fin_emit(const uint64_t* __restrict__ a,
         uint32_t lo = 0, hi = n_targets;  // last t with wb[t] <= x
         while (hi - lo > 1) {
             const uint32_t mid = (lo + hi) >> 1;
-            if (wb[mid] <= x) lo = mid; else hi = mid;
+            if (wb(mid) <= x) lo = mid; else hi = mid;
         }
         first_target[b] = lo;
     }
     __syncthreads();
-    unsigned long long n_over = 0;
+    uint32_t n_over = 0;
     for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const uint64_t base = tile * FIN_TILE + (uint64_t)w * 32 * FIN_ITEMS + lane;
-        uint64_t v[FIN_ITEMS];
-        uint32_t kmask = 0, smask = 0;  // per item: kept / run start
+        uint64_t v[FIN_ITEMS], back[FIN_ITEMS];
+        uint64_t before = (lane == 0 && base > 0 && base - 1 < n) ? a[base - 1] : SENTINEL_PAIR;
+#pragma unroll
+        for (int i = 0; i < FIN_ITEMS; ++i) {
+            const uint64_t e = base + (uint64_t)i * 32;
+            v[i] = e < n ? a[e] : SENTINEL_PAIR;
+            back[i] = e < n && e >= cap ? a[e - cap] : SENTINEL_PAIR;
+        }
+        // as fin_flags, with the predecessor from the neighbouring lane
+        uint32_t bk[FIN_ITEMS], bs[FIN_ITEMS];  // ballots: kept, run start
         uint32_t nk = 0, ns = 0;
 #pragma unroll
         for (int i = 0; i < FIN_ITEMS; ++i) {
-            bool st, kept, over;
-            fin_flags(a, n, cap, base + (uint64_t)i * 32, v[i], st, kept, over);
-            kmask |= (kept ? 1u : 0u) << i;
-            smask |= (st ? 1u : 0u) << i;
-            nk += __popc(__ballot_sync(FULL_MASK, kept));
-            ns += __popc(__ballot_sync(FULL_MASK, st));
-            n_over += over;
+            const uint64_t e = base + (uint64_t)i * 32;
+            uint64_t prev = __shfl_up_sync(FULL_MASK, v[i], 1);
+            if (lane == 0) prev = before;
+            before = __shfl_sync(FULL_MASK, v[i], 31);
+            const bool real = v[i] != SENTINEL_PAIR;
+            const uint32_t hk = hk_of(v[i]);
+            const bool st = real && (e == 0 || !same_feature(prev, hk));
+            const bool dropped = real && e >= cap && same_feature(back[i], hk);
+            // the first dropped pair of an overflowing run: the pair cap earlier starts the run
+            if (dropped && (e == cap || !same_feature(a[e - cap - 1], hk))) ++n_over;
+            bk[i] = __ballot_sync(FULL_MASK, real && !dropped);
+            bs[i] = __ballot_sync(FULL_MASK, st);
+            nk += __popc(bk[i]);
+            ns += __popc(bs[i]);
         }
         if (lane == 0) {
             wk[w] = nk;
@@ -895,37 +909,51 @@ __global__ void __launch_bounds__(BT) k_fin_emit(const uint64_t* __restrict__ a,
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < FIN_ITEMS; ++i) {
-            const bool kept = (kmask >> i) & 1u, st = (smask >> i) & 1u;
-            const uint32_t bk = __ballot_sync(FULL_MASK, kept);
-            const uint32_t bs = __ballot_sync(FULL_MASK, st);
-            const uint64_t my_k = kpos + __popc(bk & lt);
-            if (kept) {
-                const uint32_t gw = (uint32_t)v[i];
-                const uint32_t rng = gw >> bshift;  // < FIN_BUCKETS since gw < n_win
-                uint32_t lo = first_target[rng];    // last t with wb[t] <= gw lies in [lo, hi)
-                uint32_t hi = min(first_target[rng + 1] + 1, n_targets);
-                while (hi - lo > 1) {
-                    const uint32_t mid = (lo + hi) >> 1;
-                    if (wb[mid] <= gw) lo = mid; else hi = mid;
+        for (int i0 = 0; i0 < FIN_ITEMS; i0 += 4) {
+            uint32_t lo[4], hi[4];
+            bool open = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                // (a sentinel or dropped pair searches too, in bounds; its result is not used)
+                const uint32_t rng = min((uint32_t)v[i0 + u] >> bshift, FIN_BUCKETS - 1);
+                lo[u] = first_target[rng];  // last t with wb[t] <= gw lies in [lo, hi)
+                hi[u] = min(first_target[rng + 1] + 1, n_targets);
+                open |= hi[u] - lo[u] > 1;
+            }
+            while (__any_sync(FULL_MASK, open)) {
+                open = false;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (hi[u] - lo[u] > 1) {
+                        const uint32_t mid = (lo[u] + hi[u]) >> 1;
+                        if (wb(mid) <= (uint32_t)v[i0 + u]) lo[u] = mid; else hi[u] = mid;
+                        open |= hi[u] - lo[u] > 1;
+                    }
                 }
-                if (jbits)
-                    static_cast<uint32_t*>(locs)[my_k] = (lo << jbits) | (gw - wb[lo]);
-                else
-                    static_cast<uint64_t*>(locs)[my_k] = ((uint64_t)lo << 32) | (gw - wb[lo]);
             }
-            if (st) {
-                const uint64_t my_s = kidx + __popc(bs & lt);
-                khk[my_s] = hk_of(v[i]);
-                koff[my_s] = my_k;
-                kstart[my_s] = base + (uint64_t)i * 32;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = i0 + u;
+                const uint64_t my_k = kpos + __popc(bk[i] & lt);
+                if ((bk[i] >> lane) & 1u) {
+                    const uint32_t off = (uint32_t)v[i] - wb(lo[u]);
+                    if (jbits)
+                        static_cast<uint32_t*>(locs)[my_k] = (lo[u] << jbits) | off;
+                    else
+                        static_cast<uint64_t*>(locs)[my_k] = ((uint64_t)lo[u] << 32) | off;
+                }
+                if ((bs[i] >> lane) & 1u) {
+                    const uint64_t my_s = kidx + __popc(bs[i] & lt);
+                    khk[my_s] = hk_of(v[i]);
+                    koff[my_s] = my_k;
+                }
+                kpos += __popc(bk[i]);
+                kidx += __popc(bs[i]);
             }
-            kpos += __popc(bk);
-            kidx += __popc(bs);
         }
     }
-    for (int o = 16; o >= 1; o >>= 1) n_over += __shfl_xor_sync(FULL_MASK, n_over, o);
-    if (lane == 0 && n_over) atomicAdd(overflow, n_over);
+    n_over = __reduce_add_sync(FULL_MASK, n_over);
+    if (lane == 0 && n_over) atomicAdd(overflow, (unsigned long long)n_over);
 }
 
 // Pairs (h2 << 32 | global window) of a finalized layout, in layout order:
@@ -962,12 +990,21 @@ __global__ void __launch_bounds__(BT) k_exclusive_max_i64(const int64_t* __restr
                                                           uint64_t n, int64_t* total) {
     __shared__ int64_t sm[NWARP];
     int64_t carry = INT64_MIN;
-    for (uint64_t base = 0; base < n; base += BT) {
-        uint64_t e = base + threadIdx.x;
-        int64_t v = e < n ? in[e] : INT64_MIN;
+    for (uint64_t base = 0; base < n; base += BT * 8) {
+        const uint64_t e0 = base + threadIdx.x * 8;
+        int64_t v[8], m = INT64_MIN;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v[i] = e0 + i < n ? in[e0 + i] : INT64_MIN;
+            m = max(m, v[i]);
+        }
         int64_t tot;
-        int64_t ex = block_exclusive(v, (int64_t)INT64_MIN, OpMaxI(), sm, &tot);
-        if (e < n) out[e] = max(carry, ex);
+        int64_t ex = max(carry, block_exclusive(m, (int64_t)INT64_MIN, OpMaxI(), sm, &tot));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (e0 + i < n) out[e0 + i] = ex;
+            ex = max(ex, v[i]);
+        }
         carry = max(carry, tot);
     }
     if (threadIdx.x == 0) *total = carry;
@@ -994,41 +1031,88 @@ __global__ void __launch_bounds__(BT) k_tab_dispmax(const uint32_t* __restrict__
     }
 }
 
-// slot(k) = k + max(prefix, inclusive max of home - k); writes the packed
-// word (count = kept locations, koff[k + 1] - koff[k]).  A displacement beyond the word's field sets *too_far (the host then
-// retries with a larger table).
-__global__ void __launch_bounds__(BT) k_tab_emit(const uint32_t* __restrict__ khk, const uint64_t* __restrict__ koff,
+// slot(k) = k + max(prefix, inclusive max of home - k): packs the words
+// (count = kept locations, koff[k + 1] - koff[k]) and writes the table.  A
+// thread takes eight consecutive keys, so a tile needs one block-wide scan;
+// the tile's keys take consecutive slots up to the next tile's first one, and
+// the block writes that whole range, empty words included, through shared
+// memory with consecutive threads on consecutive words (the table is not
+// cleared before).  A displacement beyond the word's field sets *too_far (the
+// host then retries with a larger table).
+constexpr uint32_t TAB_CHUNK = 4096;  // slots staged at a time
+
+__global__ void __launch_bounds__(BT, 3) k_tab_emit(const uint32_t* __restrict__ khk, const uint64_t* __restrict__ koff,
                                                  uint64_t n, TableFmt fmt, const int64_t* __restrict__ tpre, uint64_t n_tiles,
-                                                 uint64_t* __restrict__ table, unsigned int* max_disp,
-                                                 unsigned int* too_far) {
+                                                 uint64_t* __restrict__ table, uint64_t table_len,
+                                                 unsigned int* max_disp, unsigned int* too_far) {
     __shared__ int64_t sm[NWARP];
-    __shared__ uint64_t smu[NWARP];
+    __shared__ __align__(16) uint64_t out[TAB_CHUNK];
+    static_assert(FIN_ITEMS == 8, "eight keys per thread");
+    uint32_t most = 0;
     for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        uint64_t base = tile * FIN_TILE;
-        int64_t carry = tpre[tile];
-        uint64_t dmax = 0;
-        for (int i = 0; i < FIN_ITEMS; ++i) {
-            uint64_t e = base + (uint64_t)i * BT + threadIdx.x;
-            bool in_range = e < n;
-            uint32_t hk = in_range ? khk[e] : 0;
-            uint64_t home = fmt.home(hk);
-            int64_t a = in_range ? (int64_t)home - (int64_t)e : INT64_MIN;
-            int64_t tot;
-            int64_t ex = block_exclusive(a, (int64_t)INT64_MIN, OpMaxI(), sm, &tot);
-            int64_t inc = max(carry, max(ex, a));
-            carry = max(carry, tot);
-            if (in_range) {
-                uint64_t slot = (uint64_t)((int64_t)e + inc);
-                const uint32_t cnt = (uint32_t)(koff[e + 1] - koff[e]);  // kept locations (<= cap)
-                const uint64_t disp = slot - home;
-                if (disp > TAB_MAX_DISP) atomicMax(too_far, 1u);
-                table[slot] = fmt.pack(koff[e], hk, (uint32_t)(disp & TAB_MAX_DISP), cnt);
-                dmax = max(dmax, disp);
+        const uint64_t first = tile * FIN_TILE;
+        const uint64_t e0 = first + threadIdx.x * FIN_ITEMS;
+        uint32_t hk[FIN_ITEMS];
+        uint64_t off[FIN_ITEMS + 1];
+        if (e0 + FIN_ITEMS <= n) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(khk + e0));
+            const uint4 y = __ldg(reinterpret_cast<const uint4*>(khk + e0) + 1);
+            hk[0] = x.x, hk[1] = x.y, hk[2] = x.z, hk[3] = x.w;
+            hk[4] = y.x, hk[5] = y.y, hk[6] = y.z, hk[7] = y.w;
+#pragma unroll
+            for (int i = 0; i < FIN_ITEMS; i += 2) {
+                const ulonglong2 z = __ldg(reinterpret_cast<const ulonglong2*>(koff + e0 + i));
+                off[i] = z.x;
+                off[i + 1] = z.y;
             }
+            off[FIN_ITEMS] = koff[e0 + FIN_ITEMS];
+        } else {
+#pragma unroll
+            for (int i = 0; i < FIN_ITEMS; ++i) hk[i] = e0 + i < n ? khk[e0 + i] : 0u;
+#pragma unroll
+            for (int i = 0; i <= FIN_ITEMS; ++i) off[i] = e0 + i <= n ? koff[e0 + i] : 0u;
         }
-        uint64_t dm = block_reduce(dmax, (uint64_t)0, OpMaxU(), smu);
-        if (threadIdx.x == 0) atomicMax(max_disp, (unsigned int)min(dm, (uint64_t)0xFFFFFFFFu));
+        int64_t m = INT64_MIN;
+#pragma unroll
+        for (int i = 0; i < FIN_ITEMS; ++i)
+            if (e0 + i < n) m = max(m, (int64_t)fmt.home(hk[i]) - (int64_t)(e0 + i));
+        int64_t tot;
+        int64_t run = max(tpre[tile], block_exclusive(m, (int64_t)INT64_MIN, OpMaxI(), sm, &tot));
+        uint64_t slot[FIN_ITEMS], word[FIN_ITEMS];
+#pragma unroll
+        for (int i = 0; i < FIN_ITEMS; ++i) {
+            const uint64_t home = fmt.home(hk[i]);
+            const bool in = e0 + i < n;
+            if (in) run = max(run, (int64_t)home - (int64_t)(e0 + i));
+            slot[i] = in ? (uint64_t)((int64_t)(e0 + i) + run) : ~0ull;
+            const uint64_t disp = in ? slot[i] - home : 0;
+            if (disp > TAB_MAX_DISP) atomicMax(too_far, 1u);
+            most = max(most, (uint32_t)min(disp, (uint64_t)0xFFFFFFFFu));
+            word[i] = fmt.pack(off[i], hk[i], (uint32_t)(disp & TAB_MAX_DISP), (uint32_t)(off[i + 1] - off[i]));
+        }
+        // the tile's slots: from its first key's (or 0) to the next tile's first key's
+        const auto first_slot = [&](uint64_t t) -> uint64_t {
+            if (t == 0) return 0;
+            if (t >= n_tiles) return table_len;
+            const uint64_t e = t * FIN_TILE;
+            return (uint64_t)((int64_t)e + max(tpre[t], (int64_t)fmt.home(khk[e]) - (int64_t)e));
+        };
+        const uint64_t s1 = first_slot(tile + 1);
+        for (uint64_t s0 = first_slot(tile); s0 < s1; s0 += TAB_CHUNK) {
+            for (uint32_t i = threadIdx.x; i < TAB_CHUNK / 2; i += BT)
+                reinterpret_cast<ulonglong2*>(out)[i] = make_ulonglong2(0, 0);
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < FIN_ITEMS; ++i)
+                if (slot[i] - s0 < TAB_CHUNK) out[slot[i] - s0] = word[i];
+            __syncthreads();
+            const uint32_t len = (uint32_t)min(s1 - s0, (uint64_t)TAB_CHUNK);
+            for (uint32_t i = threadIdx.x; i < len; i += BT) table[s0 + i] = out[i];
+            __syncthreads();
+        }
     }
+    most = __reduce_max_sync(FULL_MASK, most);
+    if (lane_id() == 0 && most) atomicMax(max_disp, most);
 }
 }  // namespace
 
@@ -1076,21 +1160,20 @@ cudaError_t finalize_pairs(const Mem& mem, const uint64_t* sorted, uint64_t n, u
         return cudaSuccess;
     }
     Tmp<unsigned char> locs(mem, n_kept * loc_bytes(jbits), s);
-    Tmp<uint64_t> koff(mem, n_keys + 1, s), kstart(mem, n_keys + 1, s);
+    Tmp<uint64_t> koff(mem, n_keys + 1, s);
     Tmp<uint32_t> khk(mem, n_keys, s);
-    if (!locs.ok() || !koff.ok() || !kstart.ok() || !khk.ok()) return cudaErrorMemoryAllocation;
+    if (!locs.ok() || !koff.ok() || !khk.ok()) return cudaErrorMemoryAllocation;
     if (n > 0) {
         // wbase in shared memory when it fits next to the range table
         const bool wb_smem = n_targets + 1 <= FIN_WB_SMEM_MAX;
         const size_t smem = (size_t)(FIN_BUCKETS + 1 + (wb_smem ? n_targets + 1 : 0)) * 4;
-        if ((e = cudaFuncSetAttribute(k_fin_emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
+        const auto kern = wb_smem ? k_fin_emit<true> : k_fin_emit<false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
         MC_LAUNCH("fin_emit", s,
-                  k_fin_emit<<<g, BT, smem, s>>>(sorted, n, cap, tkept.ptr, tkeys.ptr, tiles, wbase, n_targets, jbits,
-                                                 locs.ptr, khk.ptr, koff.ptr, kstart.ptr, ctr.ptr, wb_smem));
+                  kern<<<g, BT, smem, s>>>(sorted, n, cap, tkept.ptr, tkeys.ptr, tiles, wbase, n_targets, jbits,
+                                           locs.ptr, khk.ptr, koff.ptr, ctr.ptr));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = cudaMemcpyAsync(kstart.ptr + n_keys, &n, 8, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
         if ((e = cudaMemcpyAsync(koff.ptr + n_keys, &n_kept, 8, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
     }
     const uint64_t ktiles = (n_keys + FIN_TILE - 1) / FIN_TILE;
@@ -1115,12 +1198,12 @@ cudaError_t finalize_pairs(const Mem& mem, const uint64_t* sorted, uint64_t n, u
         const uint64_t table_len = (((last_slot + 1 > T ? last_slot + 1 : T) + 2) + 3) & ~3ull;
         Tmp<uint64_t> table(mem, table_len, s);
         if (!table.ok()) return cudaErrorMemoryAllocation;
-        if ((e = cudaMemsetAsync(table.ptr, 0, table_len * sizeof(uint64_t), s)) != cudaSuccess) return e;
+        if (n_keys == 0 && (e = cudaMemsetAsync(table.ptr, 0, table_len * sizeof(uint64_t), s)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(ctr.ptr + 1, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return e;
         if (n_keys > 0) {
             MC_LAUNCH("tab_emit", s,
                       k_tab_emit<<<grid_for(ktiles), BT, 0, s>>>(khk.ptr, koff.ptr, n_keys, fmt, kt_pre.ptr, ktiles,
-                                                                 table.ptr,
+                                                                 table.ptr, table_len,
                                                                  (unsigned int*)(ctr.ptr + 1),
                                                                  (unsigned int*)(ctr.ptr + 2)));
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
