@@ -545,7 +545,7 @@ int finalize_impl(mc_db* db, uint32_t n_lists, const uint32_t* const* keys, cons
         cudaError_t e = mc::reconstruct_pairs((const uint64_t*)db->table.p, db->table_len, db->fmt, db->locs.p,
                                               db->loc_jbits, (const uint32_t*)db->wbase.p, (uint64_t*)old.p, s);
         if (e == cudaSuccess)
-            e = mc::merge_sorted_pairs((const uint64_t*)old.p, n_old, (const uint64_t*)db->pending.p, n_new,
+            e = mc::merge_sorted_pairs(db->mem, (const uint64_t*)old.p, n_old, (const uint64_t*)db->pending.p, n_new,
                                        (uint64_t*)a.p, s);
         release(db, old);
         if (e != cudaSuccess) {

@@ -542,7 +542,10 @@ __global__ void __launch_bounds__(BT) k_radix_totals(const uint64_t* __restrict_
 // shared memory, then reads the word back; two tables alternate so that a
 // table's reset is ordered before its next use by the warp barriers of the
 // round in between) and the warp's running count of that digit.  Invalid
-// lanes carry digit 256, which is neither counted nor reset.
+// lanes carry digit 256, which is neither counted nor reset.  Bound by shared
+// memory (L1 77% busy, issue 51%); peers from eight ballots (60.8 ms for the
+// four passes of the large workload, then bound by the ALU) or match.any
+// (55.9 ms) are slower than this (45.3 ms).
 __device__ __forceinline__ uint32_t rank_round(int i, bool valid, uint32_t d, uint32_t lane, uint32_t lt,
                                                uint32_t* wcount, uint32_t* mask0, uint32_t* mask1) {
     uint32_t* mask = (i & 1) ? mask1 : mask0;
@@ -1237,8 +1240,8 @@ cudaError_t finalize_pairs(const Mem& mem, const uint64_t* sorted, uint64_t n, u
 // targets are two sorted runs; merging them gives the sorted pairs of the
 // whole database without sorting the stored ones again.  Merge path
 // (Odeh, Green, Mwassi, Shmueli, Birk 2012): a block takes 2,048
-// consecutive outputs, finds where that output range starts and ends in
-// both inputs by a binary search along the diagonals, stages the two input
+// consecutive outputs, takes where that output range starts and ends in
+// both inputs (a binary search along the diagonals, k_merge_splits), stages the two input
 // slices in shared memory, and each thread merges eight outputs.
 namespace {
 constexpr int MP_ITEMS = 8;
@@ -1256,18 +1259,26 @@ __device__ __forceinline__ uint64_t merge_split(const uint64_t* a, uint64_t na, 
     return lo;
 }
 
+// split[i] = elements of a in the first min(i * MP_TILE, na + nb) outputs.  A
+// kernel of its own, a thread per tile: searched by the merging blocks, a
+// tile waited for about 27 dependent reads before it could start (four
+// merges of 300 M pairs in all: 3.75 ms, now 0.15 + 1.71).
+__global__ void __launch_bounds__(BT) k_merge_splits(const uint64_t* __restrict__ a, uint64_t na,
+                                                     const uint64_t* __restrict__ b, uint64_t nb,
+                                                     uint64_t* __restrict__ split, uint64_t n_split) {
+    for (uint64_t i = blockIdx.x * (uint64_t)BT + threadIdx.x; i < n_split; i += (uint64_t)gridDim.x * BT)
+        split[i] = merge_split(a, na, b, nb, min(i * MP_TILE, na + nb));
+}
+
 __global__ void __launch_bounds__(BT) k_merge_path(const uint64_t* __restrict__ a, uint64_t na,
                                                    const uint64_t* __restrict__ b, uint64_t nb,
-                                                   uint64_t* __restrict__ c) {
+                                                   const uint64_t* __restrict__ splits, uint64_t* __restrict__ c) {
     __shared__ uint64_t in[MP_TILE];
     __shared__ uint64_t out[MP_TILE];
-    __shared__ uint64_t split[2];
     const uint64_t n = na + nb;
     for (uint64_t d0 = (uint64_t)blockIdx.x * MP_TILE; d0 < n; d0 += (uint64_t)gridDim.x * MP_TILE) {
         const uint64_t d1 = min(d0 + MP_TILE, n);
-        if (threadIdx.x < 2) split[threadIdx.x] = merge_split(a, na, b, nb, threadIdx.x ? d1 : d0);
-        __syncthreads();
-        const uint64_t i0 = split[0], i1 = split[1];
+        const uint64_t i0 = splits[d0 / MP_TILE], i1 = splits[d0 / MP_TILE + 1];
         const uint32_t ta = (uint32_t)(i1 - i0), tb = (uint32_t)((d1 - d0) - ta);
         for (uint32_t k = threadIdx.x; k < ta + tb; k += BT) in[k] = k < ta ? a[i0 + k] : b[(d0 - i0) + (k - ta)];
         __syncthreads();
@@ -1293,12 +1304,18 @@ __global__ void __launch_bounds__(BT) k_merge_path(const uint64_t* __restrict__ 
 }
 }  // namespace
 
-cudaError_t merge_sorted_pairs(const uint64_t* a, uint64_t na, const uint64_t* b, uint64_t nb, uint64_t* c,
-                               cudaStream_t s) {
+cudaError_t merge_sorted_pairs(const Mem& mem, const uint64_t* a, uint64_t na, const uint64_t* b, uint64_t nb,
+                               uint64_t* c, cudaStream_t s) {
     const uint64_t n = na + nb;
     if (n == 0) return cudaSuccess;
-    MC_LAUNCH("merge_path", s,
-              k_merge_path<<<grid_for((n + MP_TILE - 1) / MP_TILE, 4), BT, 0, s>>>(a, na, b, nb, c));
+    const uint64_t tiles = (n + MP_TILE - 1) / MP_TILE;
+    Tmp<uint64_t> splits(mem, tiles + 1, s);
+    if (!splits.ok()) return cudaErrorMemoryAllocation;
+    MC_LAUNCH("merge_splits", s,
+              k_merge_splits<<<grid_for((tiles + BT) / BT), BT, 0, s>>>(a, na, b, nb, splits.ptr, tiles + 1));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    MC_LAUNCH("merge_path", s, k_merge_path<<<grid_for(tiles, 6), BT, 0, s>>>(a, na, b, nb, splits.ptr, c));
     return cudaGetLastError();
 }
 

@@ -120,8 +120,8 @@ cudaError_t finalize_pairs(const Mem& mem, const uint64_t* sorted, uint64_t n, u
                            uint32_t n_targets, uint32_t jbits, FinalizeOut* out, cudaStream_t s);
 
 // c[0..na+nb) = the merge of the sorted pair runs a and b (ties from a).
-cudaError_t merge_sorted_pairs(const uint64_t* a, uint64_t na, const uint64_t* b, uint64_t nb, uint64_t* c,
-                               cudaStream_t s);
+cudaError_t merge_sorted_pairs(const Mem& mem, const uint64_t* a, uint64_t na, const uint64_t* b, uint64_t nb,
+                               uint64_t* c, cudaStream_t s);
 
 // Sharded builds (Section 4.3): distinct features of sorted pairs a[0..n)
 // (h2 keys ascending) with their counts clamped to cap; *n_keys = the
