@@ -1793,6 +1793,77 @@ __device__ __forceinline__ bool query_sort(const ClassifyDb& db, const ClassifyQ
     return true;
 }
 
+// A query of H <= 32 locations, one per lane: gather, sort, runs, scores and
+// top m stay in registers (through the shared memory of the larger ones it
+// takes twice the instructions).
+template <class LocT>
+__device__ __forceinline__ void query_small(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
+                                            const uint64_t* src, uint32_t n_list, uint32_t sws, uint32_t H,
+                                            uint32_t& distinct) {
+    const uint32_t lane = lane_id();
+    const uint32_t le = lanemask_lt() | (1u << lane);
+    const uint32_t jb = sizeof(LocT) == 8 ? 32u : db.jbits;
+    const uint32_t jmask = sizeof(LocT) == 8 ? 0xFFFFFFFFu : (1u << jb) - 1u;
+    const uint64_t e = lane < n_list ? __ldg(src + lane) : 0;  // n_list <= H: no bucket is empty
+    const uint32_t c = (uint32_t)e & 0xFFFFu;
+    uint32_t pre = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t x = __shfl_up_sync(FULL_MASK, pre, d);
+        if ((int)lane >= d) pre += x;
+    }
+    pre -= c;
+    const uint32_t starts = __reduce_or_sync(FULL_MASK, lane < n_list ? 1u << (pre & 31u) : 0u);
+    const uint64_t adj = __shfl_sync(FULL_MASK, (e >> 16) - pre, (__popc(starts & le) - 1) & 31);
+    LocT k[1] = {~(LocT)0};
+    if (lane < H) k[0] = __ldg(static_cast<const LocT*>(db.locs) + (adj + lane));
+    warp_bitonic_sort<1>(k);
+    const LocT x = k[0];
+    const LocT prev = __shfl_up_sync(FULL_MASK, x, 1);
+    const bool start = lane < H && (lane == 0 || x != prev);
+    distinct = __popc(__ballot_sync(FULL_MASK, start));
+    const uint32_t t = (uint32_t)(x >> jb), win = (uint32_t)x & jmask;
+    const LocT hi = x + min(sws ? sws - 1 : 0u, jmask - win);
+    uint32_t ub = 0;  // locations <= hi
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) {
+        const LocT v = __shfl_sync(FULL_MASK, x, ub + s - 1);
+        if (v <= hi) ub += s;
+    }
+    if (__shfl_sync(FULL_MASK, x, ub & 31u) <= hi) ++ub;
+    ub = min(ub, H);
+    uint32_t sc = start ? ub - lane : 0u;
+
+    const int m = (int)Q.m;
+    Cand mine = Cand{0, 0xFFFFFFFFu, 0, 0};
+    uint32_t label = NO_TAXON, hits = 0, top = 0xFFFFFFFFu;
+    uint64_t bar = 0;
+    for (int rd = 0; rd < m; ++rd) {
+        const uint32_t ms = __reduce_max_sync(FULL_MASK, sc);
+        if (ms == 0) break;
+        const uint32_t mt = __reduce_min_sync(FULL_MASK, sc == ms ? t : 0xFFFFFFFFu);
+        if (Q.cands) {
+            const uint32_t mj = __reduce_min_sync(FULL_MASK, sc == ms && t == mt ? win : 0xFFFFFFFFu);
+            const uint32_t l = __ffs(__ballot_sync(FULL_MASK, sc == ms && t == mt && win == mj)) - 1;
+            const uint32_t j1 = __shfl_sync(FULL_MASK, win, __shfl_sync(FULL_MASK, ub, l) - 1);
+            if ((int)lane == rd) mine = Cand{ms, mt, mj, j1};
+        }
+        if (t == mt) sc = 0;  // one candidate per target
+        if (rd == 0) {
+            hits = ms;
+            top = mt;
+            bar = (uint64_t)(100 - Q.band) * hits;
+            if (hits >= Q.hits_min) label = top < db.n_targets ? db.taxon_of_target[top] : NO_TAXON;
+            else if (!Q.cands) break;
+        } else if (hits >= Q.hits_min && 100ull * ms >= bar) {
+            label = lca2(db, label, mt < db.n_targets ? db.taxon_of_target[mt] : NO_TAXON);
+        } else if (!Q.cands) {
+            break;
+        }
+    }
+    write_result(Q, q, label, hits, top, mine);
+}
+
 // Resident CTAs per SM that the register budget of a sort-path kernel is
 // sized for.
 template <int E, class LocT>
@@ -1812,17 +1883,27 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t w = threadIdx.x >> 5;
     const SortMem<E, LocT> M(smem + w * SortMem<E, LocT>::bytes(list_cap), list_cap);
+    // the next size class, which shares no data with this one, may start
+    // while this one's last queries finish
+    asm volatile("griddepcontrol.launch_dependents;");
     const uint32_t total = total_queries(Q);
     if (q0 < total) {
         ChunkScan it = chunk_scan(min(chunk, total - q0), group_shift, group_ctr);
         uint32_t i;
         uint4 mt;
         while (next_chunk_query(it, meta, h_lo, 32u * E, last ? mid_list : nullptr, mid_n, i, mt)) {
-            sort_gather<E>(db, M, glist + (uint64_t)i * list_cap, mt.x, mt.z);
-            cp_async_wait_all();
-            __syncwarp();
+            const uint64_t* src = glist + (uint64_t)i * list_cap;
             uint32_t distinct;
-            if (!query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct)) {
+            bool done = true;
+            if (E == 8 && mt.z <= 32) {
+                query_small<LocT>(db, Q, q0 + i, src, mt.x, meta_sws(mt), mt.z, distinct);
+            } else {
+                sort_gather<E>(db, M, src, mt.x, mt.z);
+                cp_async_wait_all();
+                __syncwarp();
+                done = query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct);
+            }
+            if (!done) {
                 if (lane_id() == 0) mid_list[atomicAdd(mid_n, 1u)] = i;
             } else if (Q.counters) {  // per query: a debug call need not keep them in registers
                 Counters ctr;
@@ -1836,11 +1917,11 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
             }
         }
     }
-    // Launched as a programmatic dependent of the medium path, this kernel
-    // may run alongside it; waiting for that grid before exiting makes this
-    // kernel's completion imply the medium path's, so that later work in
-    // the stream or graph never overtakes it.  A no-op for an ordinary
-    // launch.
+    // Launched as a programmatic dependent of the medium path or of another
+    // size class, this kernel may run alongside it; waiting for that grid
+    // before exiting makes this kernel's completion imply the other's, so
+    // that later work in the stream or graph never overtakes it.  A no-op
+    // for an ordinary launch.
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -2527,14 +2608,14 @@ cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const Cl
 
 // Score of the chunk at q0.  Sort path, 32-bit locations: the largest size
 // class first (it queues the queries beyond it), then the medium path, then
-// the other classes, the most populous one (512) launched with programmatic
-// stream serialization so that it fills the SMs the medium path's few long
-// queries leave idle (they share no data: the sort kernels read the
-// lookup's outputs and write other queries' results; their groups of
-// queries come from a counter, so the CTAs that start late take fewer).
-// 64-bit locations: every class may queue queries, so the medium path comes
-// last.  Hash path: the score kernel, then the medium path for the queries
-// whose histogram did not fit.
+// the other classes, the most populous one (512) first.  Each of those is
+// launched with programmatic stream serialization, so that it fills the SMs
+// that the last queries of the kernel before leave idle (they share no data:
+// the sort kernels read the lookup's outputs and write other queries'
+// results; their groups of queries come from a counter, so the CTAs that
+// start late take fewer).  64-bit locations: every class may queue queries,
+// so the medium path comes last.  Hash path: the score kernel, then the
+// medium path for the queries whose histogram did not fit.
 cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
                          uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
@@ -2552,13 +2633,12 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
                                                       "classify_sort2048"};
     const int last = g.n_sort - 1;
     const bool narrow = db.jbits != 0;
-    const int pdl = narrow && last >= 2 ? 1 : -1;  // the class launched as the medium path's dependent
     int order[N_SORT_CLASSES + 1], n = 0;
     order[n++] = last;
     if (narrow) order[n++] = -1;  // medium path
-    if (pdl >= 0) order[n++] = pdl;
+    if (last >= 2) order[n++] = 1;
     for (int c = 0; c < last; ++c)
-        if (c != pdl) order[n++] = c;
+        if (c != 1 || last < 2) order[n++] = c;
     if (!narrow) order[n++] = -1;
     for (int k = 0; k < n; ++k) {
         const int c = order[k];
@@ -2576,7 +2656,7 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = c == pdl ? 1 : 0;
+        cfg.numAttrs = k > 0 ? 1 : 0;  // after the medium path or another class
         MC_LAUNCH(names[c], s,
                   e = cudaLaunchKernelEx(&cfg, g.kt[c], db, Q, q0, (uint32_t)sc.chunk, g.list_cap,
                                          (const uint64_t*)sc.glist, (const uint4*)sc.meta, h_lo, c == last, g.group_shift,
