@@ -1865,10 +1865,13 @@ __device__ __forceinline__ void query_small(const ClassifyDb& db, const Classify
 }
 
 // Resident CTAs per SM that the register budget of a sort-path kernel is
-// sized for.
+// sized for.  The classes are bound by issue and by the latency of the
+// gather, and more warps help up to where registers spill in the loops
+// (sort256: 319 us at 8, 300 at 10 CTAs, 64-bit locations 381 at 5, 336 at 7;
+// sort512: 3.28 ms at 8, 3.33 at 9).
 template <int E, class LocT>
 constexpr int sort_min_ctas() {
-    return sizeof(LocT) == 8 ? (E == 8 ? 5 : (E == 16 ? 4 : 2)) : (E == 8 ? 8 : (E == 16 ? 8 : (E == 32 ? 5 : 3)));
+    return sizeof(LocT) == 8 ? (E == 8 ? 7 : (E == 16 ? 4 : 2)) : (E == 8 ? 10 : (E == 16 ? 8 : (E == 32 ? 5 : 3)));
 }
 
 // Sort path over the chunk's queries with h_lo < H <= 32*E gathered
