@@ -2404,12 +2404,13 @@ using SortKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint3
 constexpr int N_SORT_CLASSES = 4;
 constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {256, 512, 1024, 2048};
 
-// Launches of at least this many queries look up with one window per lane,
-// nine queries for each of the 3,648 resident warps; with fewer, lanes stay
+// Launches of at least this many queries look up with one window per lane:
+// four to five for each of the 3,648 resident warps; with fewer, lanes stay
 // empty and one warp per query is faster.  Measured (us, per query / per
-// lane): single reads of 100, 20,000 queries 41 / 58, 50,000 90 / 77; half
-// pairs, lengths 50-300, 20,000 queries 73 / 79, 50,000 147 / 130.
-constexpr uint32_t LANES_MIN_QUERIES = 32768;
+// lane): single reads of 100, 8,000 queries 23 / 29, 20,000 42 / 38, 100,000
+// 168 / 68; half pairs, lengths 50-300, 8,000 queries 38 / 39, 20,000 73 / 65,
+// 100,000 276 / 180.
+constexpr uint32_t LANES_MIN_QUERIES = 16384;
 
 struct Geometry {
     LookupKernel kl;         // one window per warp
@@ -2490,9 +2491,11 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->grid_l = (uint32_t)std::min<uint64_t>((c + t.lookup_warps - 1) / t.lookup_warps, (uint64_t)sms * occ_l);
     g->batch_shift = 0;
     if (g->kll) {
-        // a lane per query where that still gives every resident warp some
+        // as few queries per warp as one wave of resident warps needs, up to
+        // a lane per query (half as many, in two waves: 100,000 queries 223
+        // us instead of 180)
         const uint64_t warps = (uint64_t)sms * occ_l * t.lookup_warps;
-        while (g->batch_shift < 5 && (c >> (g->batch_shift + 1)) >= warps) ++g->batch_shift;
+        while (g->batch_shift < 5 && ((c + (1u << g->batch_shift) - 1) >> g->batch_shift) > warps) ++g->batch_shift;
         const uint64_t batches = (c + (1u << g->batch_shift) - 1) >> g->batch_shift;
         g->grid_l = (uint32_t)std::min<uint64_t>((batches + t.lookup_warps - 1) / t.lookup_warps, (uint64_t)sms * occ_l);
     }
@@ -2829,7 +2832,9 @@ cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const
     if (n_kernels) *n_kernels = 0;
     if (Q.n_q == 0) return cudaSuccess;
     if (Q.n_q > sc.n_q_cap) return cudaErrorInvalidValue;
-    if (Q.n_q <= DIRECT_MAX_QUERIES && !Q.counters) {
+    // (a CTA per piece of global scratch, and at most two queries each: of an
+    // allocation-free launch, which has eight, 16 queries)
+    if (Q.n_q <= DIRECT_MAX_QUERIES && Q.n_q <= 2 * sc.large_warps && !Q.counters) {
         if ((e = launch_direct(db, Q, sc, s)) != cudaSuccess) return e;
         if (n_kernels) *n_kernels = 1;
         return cudaSuccess;

@@ -161,3 +161,47 @@ def test_wide_locations(mc):
             _check(mc, db, odb, parent, taxon, qs, m, with_cands, hits_min=2, lca_band_pct=band, max_insert=ins)
     finally:
         db.free()
+
+
+def test_few_queries_in_every_form(mc, narrow):
+    """Launches at and around the number of queries that go straight to one
+    CTA each: several batches at once, a plan, and the allocation-free call
+    (which has fewer CTAs)."""
+    import torch
+    db, odb, parent, taxon, qs = narrow
+    cls = dict(max_candidates=4, hits_min=2, lca_band_pct=20, max_insert=390)
+    cp = mc.classify_params(**cls)
+    for sizes in ([7, 0, 1, 30], [511, 1], [300, 213], [1]):
+        cuts = np.cumsum([0, *sizes])
+        parts = [(qs * 2)[a:b] for a, b in zip(cuts[:-1], cuts[1:])]
+        plan = mc.Plan(db.handle, cp, max_batches=len(parts), max_queries=int(cuts[-1]))
+        try:
+            arrs, outs, keep = [], [], []
+            for part in parts:
+                reads, roffs, qoffs = _reads(part)
+                dv = [dev(reads) if len(reads) else torch.zeros(16, dtype=torch.uint8, device="cuda"), dev(roffs), dev(qoffs)]
+                out = [torch.full((max(1, len(part)),), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
+                arrs.append(mc.batch(len(roffs) - 1, *dv, *out))
+                outs.append(out)
+                keep.append(dv)
+            for run in (lambda: mc.mc_classify_batches(db.handle, cp, arrs), lambda: plan.run(arrs)):
+                for out in outs:
+                    for o in out:
+                        o.fill_(-7)
+                run()
+                mc.mc_classify_status(db.handle)
+                for part, out in zip(parts, outs):
+                    if part:
+                        want = odb.classify(parent, taxon, *_reads(part), n_threads=8, **cls)
+                        for g, o in zip(out, want):
+                            assert (host_u32(g) == o).all()
+        finally:
+            plan.free()
+    for n in (1, 16, 17, 300):
+        reads, roffs, qoffs = _reads(qs[:n])
+        out = [torch.full((n,), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
+        mc.mc_classify_noalloc(db.handle, cp, len(roffs) - 1, dev(reads), dev(roffs), n, dev(qoffs), *out)
+        mc.mc_classify_status(db.handle)
+        want = odb.classify(parent, taxon, reads, roffs, qoffs, n_threads=8, **cls)
+        for g, o in zip(out, want):
+            assert (host_u32(g) == o).all()
