@@ -319,7 +319,8 @@ typedef struct mc_batch {
  *                by 32 bits (target << b | window) when every target and
  *                window id of the database fits 32 bits, else by 64; 1 =
  *                always 64-bit keys (hash path).
- * One warp carries one query in every kernel. */
+ * One warp carries one query on the sort and hash paths, one CTA beyond them
+ * and in launches of at most 512 queries, which ignore the shape. */
 typedef struct mc_tuning {
     uint32_t hist_slots;
     uint32_t probe_batch;

@@ -4,9 +4,9 @@
 // GB300 design.  The paper inserts each (feature, location) pair into a
 // multi-bucket hash table with warp-aggregated atomics.  Here the build is
 // organised around streaming HBM passes instead of random-sector updates:
-//   1. sketch + emit: one warp per window computes its sketch (shared with
-//      the query path, mc_sketch.cuh) and writes (h2(feature) << 32 |
-//      global window) pairs in window order;
+//   1. sketch + emit: a warp sketches 32 windows at a time, one per lane
+//      (shared with the query path, mc_sketch.cuh), and writes (h2(feature)
+//      << 32 | global window) pairs in window order;
 //   2. a stable LSD radix sort (4 single-pass digits of 8 bits over the
 //      upper word) groups the pairs by feature while keeping them in window order,
 //      which is (target, window) order, so every bucket comes out sorted;
@@ -259,9 +259,10 @@ __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq
 // short for a window lie between them and spread the 32 windows over more
 // bytes than the staging area holds, the windows that fit are taken first.
 // A window that lane_sketch does not settle is sketched by the whole warp.
-// Bound by the integer ALU (half the issue rate): 14.3 Gbp of the large
-// workload take 22.4 ms (127 M windows of 113 k-mers), against 64.5 ms with
-// one warp per window; 25.9, 23.6 and 22.4 ms at 4, 5 and 6 CTAs per SM.
+// Bound by the integer ALU (74-80% busy, half the issue rate; 118 warp
+// instructions per window): 14.3 Gbp of the large workload take 20.5 ms (127 M
+// windows of 113 k-mers), against 64.5 ms with one warp per window.  Six CTAs
+// per SM: 5% and 15% faster than five and four.
 constexpr uint32_t EMIT_CAP = 48;  // candidates per lane
 __host__ __device__ inline uint32_t emit_stage_words(const SketchParams& p) {
     return (31 * p.stride + p.w + 30) / 16 + 2;
@@ -835,8 +836,9 @@ __global__ void __launch_bounds__(BT) k_fin_count(const uint64_t* __restrict__ a
 // wbase (n_targets + 1 words) is copied to shared memory too.
 // A thread's items are searched four at a time, one step of each per round,
 // so that their reads overlap, and a pair's predecessor comes from the lane
-// before it.  Bound by latency and issue (the pairs are read and the
-// locations written once, 28 GB on the large workload, 4 ms).
+// before it.  Bound by the ALU (70%) and issue (69%), about 130 instructions
+// per 32 pairs: large workload 13.3 ms (16.0 with one search after the other),
+// where its bytes, 28 GB, take 4.
 template <bool WB>
 __global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__ a, uint64_t n, uint32_t cap,
                                                     const uint64_t* __restrict__ tkept, const uint64_t* __restrict__ tkeys,
@@ -1040,7 +1042,8 @@ __global__ void __launch_bounds__(BT) k_tab_dispmax(const uint32_t* __restrict__
 // the tile's keys take consecutive slots up to the next tile's first one, and
 // the block writes that whole range, empty words included, through shared
 // memory with consecutive threads on consecutive words (the table is not
-// cleared before).  A displacement beyond the word's field sets *too_far (the
+// cleared before): 2.36 ms for the 2^30 slots of the large database, where
+// clearing (1.3 ms) and single words in their places took 5.2.  A displacement beyond the word's field sets *too_far (the
 // host then retries with a larger table).
 constexpr uint32_t TAB_CHUNK = 4096;  // slots staged at a time
 

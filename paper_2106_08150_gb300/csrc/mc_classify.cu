@@ -4,23 +4,22 @@
 // GB300 design.  The paper runs the query as a pipeline of kernels with
 // global-memory hand-offs: sketch+lookup, compaction, a segmented sort
 // (about half of its query time, Section 6.4) and a top-candidate kernel.
-// Here one warp carries a whole query (a read or a read pair) through all
-// steps without leaving the SM:
-//   1. sketch every window of every mate (mc_sketch.cuh) and look each
-//      feature up in the feature table (one 16-byte probe, Section 5.3);
-//   2. gather the bucket locations into a per-warp hash histogram in shared
-//      memory, location -> hit count (the window count statistic of
-//      Section 4.2, replacing compaction + segmented sort + run-length
-//      accumulation of Sections 5.4-5.6: order does not matter for counts);
-//   3. score every distinct location (t, j0) as the sum of counts of
-//      (t, j0 .. j0+sws-1) by histogram lookups (Section 5.6 sliding window);
-//   4. keep per-lane top-m lists with one candidate per target, merge them
-//      with warp shuffles (Section 5.6), and label the query by its top
-//      target or the LCA of the close candidates via the lineage table.
-// Queries whose histogram does not fit the shared-memory table (rare) are
-// queued and processed by a second kernel whose warps use a larger table in
-// global scratch memory.  Both paths run the same code, so the result does
-// not depend on the path.
+// Here a launch set has a lookup kernel and scoring kernels:
+//   1. lookup: every window of every mate is sketched (mc_sketch.cuh; one
+//      window per lane in large launches, one per warp in small ones) and
+//      each feature looked up in the feature table (one 16-byte probe,
+//      Section 5.3); a query's found buckets go to its list;
+//   2. sort path, one warp per query, in size classes: the bucket locations
+//      are gathered, those that cannot reach the label's threshold dropped by
+//      a count per (target, window block), the rest sorted in registers; runs
+//      of equal locations give the window count statistic (Section 4.2),
+//      index differences the sliding-window scores (Section 5.6), warp
+//      arg-max rounds the top candidates, labelled by the top target or the
+//      LCA of the close candidates via the lineage table;
+//   3. medium and large paths, one CTA per query, for more locations, windows
+//      or bases; launches of a few queries go straight to the large path.
+// The hash path (a tuning choice) counts locations in a per-warp shared-memory
+// histogram instead of sorting them.  Every path gives the same results.
 #include <algorithm>
 #include <type_traits>
 

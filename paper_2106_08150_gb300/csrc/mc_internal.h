@@ -224,7 +224,7 @@ struct ClassifyScratch {
     uint4* meta;           // per query of a chunk
     uint32_t* mid;         // medium-path queue of a chunk
     uint64_t* glist;       // bucket lists of a chunk
-    unsigned char* large;  // large-path working memory
+    unsigned char* large;  // large-path working memory: large_warps pieces, one per CTA
     uint32_t n_q_cap, chunk, large_warps;
 };
 uint32_t classify_default_large_warps();

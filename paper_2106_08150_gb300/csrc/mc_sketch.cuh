@@ -285,7 +285,7 @@ __device__ __forceinline__ void warp_sketch_multi(const uint8_t* const (&seq)[NW
 // as 2-bit codes.  What it saves over one warp per window: a k-mer is one
 // funnel shift of two 32-bit words (16 bases) and its reverse complement
 // another (no shuffles, no 64-bit arithmetic), and the selection sorts in
-// registers without cross-lane steps, so that a window costs about 130 warp
+// registers without cross-lane steps, so that a window costs about 120 warp
 // instructions instead of about 500.  What it needs: 32 windows to fill the
 // warp, and s <= 16.
 
