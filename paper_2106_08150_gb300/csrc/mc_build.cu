@@ -837,8 +837,8 @@ __global__ void __launch_bounds__(BT) k_fin_count(const uint64_t* __restrict__ a
 // A thread's items are searched four at a time, one step of each per round,
 // so that their reads overlap, and a pair's predecessor comes from the lane
 // before it.  Bound by the ALU (70%) and issue (69%), about 130 instructions
-// per 32 pairs: large workload 13.3 ms (16.0 with one search after the other),
-// where its bytes, 28 GB, take 4.
+// per 32 pairs: large workload 12.9 ms (16.0 with one search after the other
+// and whole pairs compared instead of keys), where its bytes, 28 GB, take 4.
 template <bool WB>
 __global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__ a, uint64_t n, uint32_t cap,
                                                     const uint64_t* __restrict__ tkept, const uint64_t* __restrict__ tkeys,
@@ -874,27 +874,36 @@ __global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__
     uint32_t n_over = 0;
     for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const uint64_t base = tile * FIN_TILE + (uint64_t)w * 32 * FIN_ITEMS + lane;
-        uint64_t v[FIN_ITEMS], back[FIN_ITEMS];
-        uint64_t before = (lane == 0 && base > 0 && base - 1 < n) ? a[base - 1] : SENTINEL_PAIR;
+        uint64_t v[FIN_ITEMS];
+        uint32_t back[FIN_ITEMS];  // key of the pair cap places earlier
+        const uint32_t* keys = reinterpret_cast<const uint32_t*>(a) + 1;  // key of pair e at keys[2 e]
+        const uint64_t lead = base - lane;
+        const bool deep = lead >= cap;  // every item has a pair cap places earlier
 #pragma unroll
         for (int i = 0; i < FIN_ITEMS; ++i) {
             const uint64_t e = base + (uint64_t)i * 32;
             v[i] = e < n ? a[e] : SENTINEL_PAIR;
-            back[i] = e < n && e >= cap ? a[e - cap] : SENTINEL_PAIR;
+            back[i] = e < n && (deep || e >= cap) ? keys[2 * (e - cap)] : 0u;
         }
-        // as fin_flags, with the predecessor from the neighbouring lane
+        // As fin_flags, on the keys alone (32 bits), with the predecessor from
+        // the neighbouring lane.  A sentinel's key is all ones, which a
+        // feature may have too: those look at the whole pair.
+        uint32_t before = lead > 0 && lead - 1 < n ? keys[2 * (lead - 1)] : 0u;
         uint32_t bk[FIN_ITEMS], bs[FIN_ITEMS];  // ballots: kept, run start
         uint32_t nk = 0, ns = 0;
 #pragma unroll
         for (int i = 0; i < FIN_ITEMS; ++i) {
             const uint64_t e = base + (uint64_t)i * 32;
-            uint64_t prev = __shfl_up_sync(FULL_MASK, v[i], 1);
-            if (lane == 0) prev = before;
-            before = __shfl_sync(FULL_MASK, v[i], 31);
-            const bool real = v[i] != SENTINEL_PAIR;
             const uint32_t hk = hk_of(v[i]);
-            const bool st = real && (e == 0 || !same_feature(prev, hk));
-            const bool dropped = real && e >= cap && same_feature(back[i], hk);
+            uint32_t prev = __shfl_up_sync(FULL_MASK, hk, 1);
+            if (lane == 0) prev = before;
+            before = __shfl_sync(FULL_MASK, hk, 31);
+            bool real = true, st = e == 0 || prev != hk, dropped = (deep || e >= cap) && back[i] == hk;
+            if (hk == 0xFFFFFFFFu) {
+                real = v[i] != SENTINEL_PAIR;
+                st = real && (e == 0 || !same_feature(a[e - 1], hk));
+                dropped = real && e >= cap && same_feature(a[e - cap], hk);
+            }
             // the first dropped pair of an overflowing run: the pair cap earlier starts the run
             if (dropped && (e == cap || !same_feature(a[e - cap - 1], hk))) ++n_over;
             bk[i] = __ballot_sync(FULL_MASK, real && !dropped);
@@ -913,6 +922,7 @@ __global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__
             kidx += wsx[i];
         }
         __syncthreads();
+        uint32_t n_k = 0, n_s = 0;
 #pragma unroll
         for (int i0 = 0; i0 < FIN_ITEMS; i0 += 4) {
             uint32_t lo[4], hi[4];
@@ -939,21 +949,21 @@ __global__ void __launch_bounds__(BT, 4) k_fin_emit(const uint64_t* __restrict__
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = i0 + u;
-                const uint64_t my_k = kpos + __popc(bk[i] & lt);
+                const uint32_t my_k = n_k + __popc(bk[i] & lt);  // within the warp's pairs
                 if ((bk[i] >> lane) & 1u) {
                     const uint32_t off = (uint32_t)v[i] - wb(lo[u]);
                     if (jbits)
-                        static_cast<uint32_t*>(locs)[my_k] = (lo[u] << jbits) | off;
+                        (static_cast<uint32_t*>(locs) + kpos)[my_k] = (lo[u] << jbits) | off;
                     else
-                        static_cast<uint64_t*>(locs)[my_k] = ((uint64_t)lo[u] << 32) | off;
+                        (static_cast<uint64_t*>(locs) + kpos)[my_k] = ((uint64_t)lo[u] << 32) | off;
                 }
                 if ((bs[i] >> lane) & 1u) {
-                    const uint64_t my_s = kidx + __popc(bs[i] & lt);
-                    khk[my_s] = hk_of(v[i]);
-                    koff[my_s] = my_k;
+                    const uint32_t my_s = n_s + __popc(bs[i] & lt);
+                    (khk + kidx)[my_s] = hk_of(v[i]);
+                    (koff + kidx)[my_s] = kpos + my_k;
                 }
-                kpos += __popc(bk[i]);
-                kidx += __popc(bs[i]);
+                n_k += __popc(bk[i]);
+                n_s += __popc(bs[i]);
             }
         }
     }
