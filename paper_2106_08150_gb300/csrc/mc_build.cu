@@ -264,13 +264,15 @@ __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq
 // windows of 113 k-mers), against 64.5 ms with one warp per window.  Six CTAs
 // per SM: 5% and 15% faster than five and four.
 constexpr uint32_t EMIT_CAP = 48;  // candidates per lane
-__host__ __device__ inline uint32_t emit_stage_words(const SketchParams& p) {
+__host__ __device__ constexpr uint32_t emit_stage_words(const SketchParams& p) {
     return (31 * p.stride + p.w + 30) / 16 + 2;
 }
-__host__ __device__ inline size_t emit_warp_bytes(const SketchParams& p) {
+__host__ __device__ constexpr size_t emit_warp_bytes(const SketchParams& p) {
     const size_t words = emit_stage_words(p);
     return words * 4 + ((words * 2 + 3) & ~(size_t)3) + ls_cand_words(EMIT_CAP) * 4;
 }
+// The parameters that need most: windows of 512 bases without overlap.
+constexpr SketchParams EMIT_LARGEST{1, LS_MAX_S, 512, 512};
 constexpr int EMIT_WARPS = 4;
 constexpr int EMIT_CTAS = 6;  // resident per SM: 80 registers, 34 KB of shared memory each
 
@@ -422,7 +424,7 @@ cudaError_t launch_sketch(const SketchParams& p, uint32_t n_seq, const uint8_t* 
                             : r == 8 ? (k16 ? k_sketch_lanes<8, 16, EMIT> : k_sketch_lanes<8, 0, EMIT>)
                                      : (k16 ? k_sketch_lanes<16, 16, EMIT> : k_sketch_lanes<16, 0, EMIT>);
         const size_t smem = EMIT_WARPS * emit_warp_bytes(p);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, EMIT_WARPS * emit_warp_bytes(EMIT_LARGEST));
         if (e != cudaSuccess) return e;
         // rounds of 32 windows per task: 16 where there are windows enough
         // for every resident warp, fewer in small calls
@@ -1184,8 +1186,7 @@ cudaError_t finalize_pairs(const Mem& mem, const uint64_t* sorted, uint64_t n, u
         const bool wb_smem = n_targets + 1 <= FIN_WB_SMEM_MAX;
         const size_t smem = (size_t)(FIN_BUCKETS + 1 + (wb_smem ? n_targets + 1 : 0)) * 4;
         const auto kern = wb_smem ? k_fin_emit<true> : k_fin_emit<false>;
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = allow_smem(kern, (size_t)(FIN_BUCKETS + 1 + (wb_smem ? FIN_WB_SMEM_MAX : 0)) * 4)) != cudaSuccess) return e;
         MC_LAUNCH("fin_emit", s,
                   kern<<<g, BT, smem, s>>>(sorted, n, cap, tkept.ptr, tkeys.ptr, tiles, wbase, n_targets, jbits,
                                            locs.ptr, khk.ptr, koff.ptr, ctr.ptr));

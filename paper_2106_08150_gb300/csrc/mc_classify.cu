@@ -35,6 +35,7 @@ constexpr int LK_WARPS = 8;                  // warps per CTA (lookup path)
 constexpr int WIN_A = 8;                     // windows per query on the shared-memory path
 constexpr uint32_t KB_SLOTS = 1u << 16;      // large-path histogram slots per warp
 constexpr uint32_t LIST_B = MC_MAX_QUERY_WINDOWS * MAX_S;
+constexpr uint32_t LIST_CAP_MAX = WIN_A * MAX_S;  // bucket list of a query of the lookup kernels, any sketch size
 constexpr int B_WARPS_PER_SM = 2;  // large-path CTAs per SM, one piece of global scratch each
 constexpr uint32_t MED_DISTINCT = 1536;      // distinct locations of a query on the medium path
 constexpr int SK_NW = 2;  // windows sketched together
@@ -2430,6 +2431,8 @@ struct Geometry {
 // Resident CTAs per SM of a kernel, remembered per thread: the query takes
 // several microseconds, and a call that classifies a handful of queries makes
 // five of them.  A function of the kernel, the launch shape and the device.
+// (A fixed array: nothing is allocated, and a thread that uses more shapes
+// than it holds asks again for the others.)
 cudaError_t resident_ctas(const void* kernel, uint32_t threads, size_t smem, int dev, int* out) {
     struct Known {
         const void* kernel;
@@ -2437,14 +2440,18 @@ cudaError_t resident_ctas(const void* kernel, uint32_t threads, size_t smem, int
         uint32_t threads;
         int dev, ctas;
     };
-    thread_local std::vector<Known> known;
-    for (const Known& k : known)
+    constexpr int MOST = 64;
+    thread_local Known known[MOST];
+    thread_local int n_known = 0;
+    for (int i = 0; i < n_known; ++i) {
+        const Known& k = known[i];
         if (k.kernel == kernel && k.smem == smem && k.threads == threads && k.dev == dev) {
             *out = k.ctas;
             return cudaSuccess;
         }
+    }
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, (int)threads, smem);
-    if (e == cudaSuccess) known.push_back(Known{kernel, smem, threads, dev, *out});
+    if (e == cudaSuccess && n_known < MOST) known[n_known++] = Known{kernel, smem, threads, dev, *out};
     return e;
 }
 
@@ -2465,20 +2472,20 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     const size_t blk = db.jbits ? sizeof(BlockMem<uint32_t>) : sizeof(BlockMem<uint64_t>);
     g->smem_b = blk;
     g->smem_m = blk;
-    if ((e = cudaFuncSetAttribute(g->km, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_m)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(g->kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_b)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(g->km, g->smem_m)) != cudaSuccess) return e;
+    if ((e = allow_smem(g->kb, g->smem_b)) != cudaSuccess) return e;
     g->grid_m = std::min<uint32_t>((uint32_t)sms * 2, std::max<uint32_t>(sc.chunk, 1));
     g->threads_l = t.lookup_warps * 32;
     g->threads_s = t.score_warps * 32;
-    g->smem_l = t.lookup_warps * (g->kll ? sizeof(LookupLanesMem) : lookup_warp_bytes(g->list_cap));
-    g->smem_s = t.score_warps * (compact ? scratch_bytes<uint16_t, uint32_t>(t.hist_slots, g->list_cap, 0, 0)
-                                         : scratch_bytes<uint16_t, uint64_t>(t.hist_slots, g->list_cap, 0, 0));
-    if ((e = cudaFuncSetAttribute(kl_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_l)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(g->ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_s)) != cudaSuccess)
-        return e;
+    const auto lookup_bytes = [&](uint32_t lc) { return g->kll ? sizeof(LookupLanesMem) : lookup_warp_bytes(lc); };
+    const auto score_bytes = [&](uint32_t lc) {
+        return compact ? scratch_bytes<uint16_t, uint32_t>(t.hist_slots, lc, 0, 0)
+                       : scratch_bytes<uint16_t, uint64_t>(t.hist_slots, lc, 0, 0);
+    };
+    g->smem_l = t.lookup_warps * lookup_bytes(g->list_cap);
+    g->smem_s = t.score_warps * score_bytes(g->list_cap);
+    if ((e = allow_smem(kl_any, LK_WARPS * lookup_bytes(LIST_CAP_MAX))) != cudaSuccess) return e;
+    if ((e = allow_smem(g->ks, CLS_WARPS * score_bytes(LIST_CAP_MAX))) != cudaSuccess) return e;
     int occ_l = 1, occ_s = 1;
     if ((e = resident_ctas(kl_any, g->threads_l, g->smem_l, dev, &occ_l)) != cudaSuccess)
         return e;
@@ -2511,12 +2518,14 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
             compact ? k_classify_sort<16, uint32_t> : k_classify_sort<16, uint64_t>,
             compact ? k_classify_sort<32, uint32_t> : k_classify_sort<32, uint64_t>,
             compact ? k_classify_sort<64, uint32_t> : nullptr};
-        const uint32_t lc = g->list_cap;
-        const size_t bytes[N_SORT_CLASSES] = {
-            compact ? SortMem<8, uint32_t>::bytes(lc) : SortMem<8, uint64_t>::bytes(lc),
-            compact ? SortMem<16, uint32_t>::bytes(lc) : SortMem<16, uint64_t>::bytes(lc),
-            compact ? SortMem<32, uint32_t>::bytes(lc) : SortMem<32, uint64_t>::bytes(lc),
-            compact ? SortMem<64, uint32_t>::bytes(lc) : 0};
+        const auto bytes = [&](int c2, uint32_t lc) {
+            const size_t b[N_SORT_CLASSES] = {
+                compact ? SortMem<8, uint32_t>::bytes(lc) : SortMem<8, uint64_t>::bytes(lc),
+                compact ? SortMem<16, uint32_t>::bytes(lc) : SortMem<16, uint64_t>::bytes(lc),
+                compact ? SortMem<32, uint32_t>::bytes(lc) : SortMem<32, uint64_t>::bytes(lc),
+                compact ? SortMem<64, uint32_t>::bytes(lc) : 0};
+            return SORT_WARPS * b[c2];
+        };
         const uint32_t largest = compact ? t.sort_max : std::min(t.sort_max, 1024u);  // 64-bit keys: registers
         // groups of 32 queries where every resident warp gets several,
         // smaller ones in small launches, down to one query per warp
@@ -2524,10 +2533,8 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
         while (g->group_shift < 5 && (c >> (g->group_shift + 1)) >= 4 * warps) ++g->group_shift;
         for (int c2 = 0; c2 < N_SORT_CLASSES && SORT_CLASS_MAX[c2] <= largest; ++c2) {
             g->kt[c2] = kts[c2];
-            g->smem_t[c2] = SORT_WARPS * bytes[c2];
-            if ((e = cudaFuncSetAttribute(kts[c2], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_t[c2])) !=
-                cudaSuccess)
-                return e;
+            g->smem_t[c2] = bytes(c2, g->list_cap);
+            if ((e = allow_smem(kts[c2], bytes(c2, LIST_CAP_MAX))) != cudaSuccess) return e;
             int occ_t = 1;
             if ((e = resident_ctas((const void*)kts[c2], SORT_WARPS * 32, g->smem_t[c2], dev, &occ_t)) !=
                 cudaSuccess)
@@ -2602,7 +2609,7 @@ constexpr uint32_t DIRECT_MAX_QUERIES = 512;
 cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc, cudaStream_t s) {
     const LargeKernel kb = pick_large(db);
     const size_t smem = db.jbits ? sizeof(BlockMem<uint32_t>) : sizeof(BlockMem<uint64_t>);
-    cudaError_t e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kb, smem);
     if (e != cudaSuccess) return e;
     const uint32_t grid = std::max<uint32_t>(1, std::min(sc.large_warps, Q.n_q));
     MC_LAUNCH("classify_large", s,

@@ -26,6 +26,16 @@ struct TraceScope {
         ::mc::note_launch(stream);                  \
     } while (0)
 
+// Allows launches of `kernel` up to `most` bytes of dynamic shared memory.
+// The limit belongs to the kernel, and calls of other threads launch it too,
+// so `most` is what the kernel's largest launch needs, whatever this call's
+// parameters: every call sets the same value, and none lowers it under
+// another's launch.
+template <class Kernel>
+inline cudaError_t allow_smem(Kernel kernel, size_t most) {
+    return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Device memory through the database's allocator (stream-ordered).
 struct Mem {
     mc_allocator a;
