@@ -347,7 +347,9 @@ int mc_classify_batches(const mc_db* db, const mc_classify_params* params, const
 
 /* A reusable classification plan: scratch memory for up to max_queries
  * queries in up to max_batches batches, and a CUDA graph of the whole
- * launch set, captured once.  mc_plan_run replays the graph for a new set
+ * launch set, captured once (for runs of few queries beside the plan's
+ * capacity, graphs of their own, captured with the first such run).
+ * mc_plan_run replays the graph for a new set
  * of batches: it copies the batch descriptors (host, n_batches) to the
  * device and launches the graph on `stream`.  A plan is re-captured
  * automatically when its database has been finalized again since.  Runs of
@@ -358,7 +360,7 @@ typedef struct mc_plan mc_plan;
 int mc_plan_create(const mc_db* db, const mc_classify_params* params, const mc_tuning* tuning,
                    uint32_t max_batches, uint32_t max_queries, mc_plan** out);
 int mc_plan_run(mc_plan* plan, uint32_t n_batches, const mc_batch* batches, void* stream);
-int mc_plan_kernels(const mc_plan* plan);  /* kernel launches per run (graph kernel nodes) */
+int mc_plan_kernels(const mc_plan* plan);  /* kernel launches (graph kernel nodes) of a full run */
 void mc_plan_free(mc_plan* plan);
 
 /* Autotuner: times every lookup setting (probe_batch x lookup_warps) and

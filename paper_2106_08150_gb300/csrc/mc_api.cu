@@ -1175,30 +1175,39 @@ struct mc_plan {
     mc::ClassifyScratch sc{};
     unsigned char* host = nullptr;  // pinned image of the descriptors
     cudaStream_t cap = nullptr;     // capture stream
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    // The launch set for at most n_q queries.  A run takes the smallest that
+    // holds its queries; the largest is captured with the plan, the others on
+    // their first use.
+    struct Set {
+        uint32_t n_q = 0;
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        uint64_t epoch = ~0ull;
+        int n_kernels = 0;
+    };
+    Set sets[mc::CLASSIFY_MAX_SIZES];
+    int n_sets = 0;
     cudaEvent_t copied = nullptr;   // the descriptor copy of the last run is done
     cudaEvent_t done = nullptr;     // the last run is done
-    uint64_t epoch = ~0ull;
-    int n_kernels = 0;
 };
 
 namespace {
 
-void plan_drop_graph(mc_plan* p) {
-    if (p->exec) cudaGraphExecDestroy(p->exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
-    p->exec = nullptr;
-    p->graph = nullptr;
+void plan_drop_graph(mc_plan::Set& set) {
+    if (set.exec) cudaGraphExecDestroy(set.exec);
+    if (set.graph) cudaGraphDestroy(set.graph);
+    set.exec = nullptr;
+    set.graph = nullptr;
+    set.epoch = ~0ull;
 }
 
-int plan_capture(mc_plan* p) {
-    plan_drop_graph(p);
+int plan_capture(mc_plan* p, mc_plan::Set& set) {
+    plan_drop_graph(set);
     const mc_db* db = p->db;
     const mc::ClassifyDb cdb = db_view(db);
     const uint32_t* bhdr = (const uint32_t*)p->desc.p;
     const mc::BatchDesc* d = (const mc::BatchDesc*)((unsigned char*)p->desc.p + desc_offset(p->max_batches));
-    const mc::ClassifyQuery q = batch_query(db, &p->params, p->max_queries, d, bhdr);
+    const mc::ClassifyQuery q = batch_query(db, &p->params, set.n_q, d, bhdr);
     MC_CU(cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal));
     int nk = 0;
     cudaError_t e = mc::classify_enqueue(cdb, q, p->tuning, p->sc, p->cap, &nk);
@@ -1209,14 +1218,15 @@ int plan_capture(mc_plan* p) {
         cudaGetLastError();
         return cuda_fail(e != cudaSuccess ? e : e2, "mc_plan: capture");
     }
-    p->graph = g;
-    e = cudaGraphInstantiate(&p->exec, g, 0);
+    set.graph = g;
+    e = cudaGraphInstantiate(&set.exec, g, 0);
     if (e != cudaSuccess) {
-        plan_drop_graph(p);
+        set.exec = nullptr;
+        plan_drop_graph(set);
         return cuda_fail(e, "mc_plan: instantiate");
     }
-    p->n_kernels = nk;
-    p->epoch = db->epoch;
+    set.n_kernels = nk;
+    set.epoch = db->epoch;
     return MC_OK;
 }
 
@@ -1308,7 +1318,10 @@ int mc_plan_create(const mc_db* db, const mc_classify_params* params, const mc_t
         return bail(cuda_fail(e, "mc_plan_create: event"));
     // the allocations above are stream-ordered on the database stream
     if ((e = cudaStreamSynchronize(db->stream)) != cudaSuccess) return bail(cuda_fail(e, "mc_plan_create"));
-    if ((rc = plan_capture(p))) return bail(rc);
+    uint32_t sizes[mc::CLASSIFY_MAX_SIZES];
+    p->n_sets = mc::classify_set_sizes(p->sc, sizes);
+    for (int i = 0; i < p->n_sets; ++i) p->sets[i].n_q = sizes[i];
+    if ((rc = plan_capture(p, p->sets[p->n_sets - 1]))) return bail(rc);
     *out = p;
     return MC_OK;
 }
@@ -1322,15 +1335,18 @@ int mc_plan_run(mc_plan* p, uint32_t n_batches, const mc_batch* batches, void* s
     const mc_db* db = p->db;
     if (!db->has_table || db->dirty) return fail(MC_ERR_STATE, "mc_plan_run: database has pending additions");
     int rc;
-    if (db->epoch != p->epoch && (rc = plan_capture(p))) return rc;
-    // the previous run's descriptor copy must be done before the image is rewritten
-    MC_CU(cudaEventSynchronize(p->copied));
     std::vector<unsigned char> img(desc_bytes(n_batches));
     uint64_t total = 0;
     if ((rc = fill_batches(n_batches, batches, img.data(), &total))) return rc;
     if (total > p->max_queries)
         return fail(MC_ERR_CAPACITY, "mc_plan_run: %llu queries, plan holds %u", (unsigned long long)total,
                     p->max_queries);
+    int i = 0;
+    while (total > p->sets[i].n_q) ++i;  // the last holds max_queries
+    mc_plan::Set& set = p->sets[i];
+    if (db->epoch != set.epoch && (rc = plan_capture(p, set))) return rc;
+    // the previous run's descriptor copy must be done before the image is rewritten
+    MC_CU(cudaEventSynchronize(p->copied));
     // the plan's image layout has its descriptors after max_batches header words
     uint32_t* hdr = reinterpret_cast<uint32_t*>(p->host);
     std::memcpy(hdr, img.data(), (size_t)(n_batches + 3) * 4);
@@ -1340,19 +1356,19 @@ int mc_plan_run(mc_plan* p, uint32_t n_batches, const mc_batch* batches, void* s
     MC_CU(cudaStreamWaitEvent(s, db->ready, 0));
     MC_CU(cudaMemcpyAsync(p->desc.p, p->host, desc_bytes(p->max_batches), cudaMemcpyHostToDevice, s));
     MC_CU(cudaEventRecord(p->copied, s));
-    MC_CU(cudaGraphLaunch(p->exec, s));
+    MC_CU(cudaGraphLaunch(set.exec, s));
     MC_CU(cudaEventRecord(p->done, s));
-    mc::note_launches((uint64_t)p->n_kernels);
+    mc::note_launches((uint64_t)set.n_kernels);
     MC_CU(note_use(db, s));
     return MC_OK;
 }
 
-int mc_plan_kernels(const mc_plan* p) { return p ? p->n_kernels : 0; }
+int mc_plan_kernels(const mc_plan* p) { return p ? p->sets[p->n_sets - 1].n_kernels : 0; }
 
 void mc_plan_free(mc_plan* p) {
     if (!p) return;
     if (p->done) cudaEventSynchronize(p->done);
-    plan_drop_graph(p);
+    for (mc_plan::Set& set : p->sets) plan_drop_graph(set);
     mc_db* mdb = const_cast<mc_db*>(p->db);
     release(mdb, p->scratch);
     release(mdb, p->desc);

@@ -2606,6 +2606,10 @@ cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const Classif
 // 115 us this way and 61 the other (reads of 100), so the line lies between.
 constexpr uint32_t DIRECT_MAX_QUERIES = 512;
 
+// (a CTA per piece of global scratch, and at most two queries each: of an
+// allocation-free launch, which has eight, 16 queries)
+uint32_t direct_max(const ClassifyScratch& sc) { return std::min(DIRECT_MAX_QUERIES, 2 * sc.large_warps); }
+
 cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc, cudaStream_t s) {
     const LargeKernel kb = pick_large(db);
     const size_t smem = db.jbits ? sizeof(BlockMem<uint32_t>) : sizeof(BlockMem<uint64_t>);
@@ -2831,16 +2835,31 @@ ClassifyScratch classify_scratch_carve(unsigned char* base, uint32_t n_q_cap, ui
     return sc;
 }
 
-cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const Tuning& t, const ClassifyScratch& sc,
-                             cudaStream_t s, int* n_kernels) {
+int classify_set_sizes(const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]) {
+    int n = 0;
+    const auto add = [&](uint32_t most) {
+        if (most < sc.n_q_cap) sizes[n++] = most;
+    };
+    add(direct_max(sc));
+    add(LANES_MIN_QUERIES - 1);
+    // from there on shapes change every doubling: the lookup's queries per warp
+    // at 8 and 16 times its 3,648 resident warps (the sizes lie just under
+    // those), the sort path's up to 32 queries per group at half a million
+    for (uint32_t most = 28 << 10; most < CHUNK; most *= 2) add(most);
+    sizes[n++] = sc.n_q_cap;
+    return n;
+}
+
+cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const Tuning& t,
+                             const ClassifyScratch& scratch, cudaStream_t s, int* n_kernels) {
     cudaError_t e;
     int n = 0;
     if (n_kernels) *n_kernels = 0;
     if (Q.n_q == 0) return cudaSuccess;
-    if (Q.n_q > sc.n_q_cap) return cudaErrorInvalidValue;
-    // (a CTA per piece of global scratch, and at most two queries each: of an
-    // allocation-free launch, which has eight, 16 queries)
-    if (Q.n_q <= DIRECT_MAX_QUERIES && Q.n_q <= 2 * sc.large_warps && !Q.counters) {
+    if (Q.n_q > scratch.n_q_cap) return cudaErrorInvalidValue;
+    ClassifyScratch sc = scratch;
+    sc.chunk = std::min(sc.chunk, Q.n_q);  // the launch's shape follows its queries, not its scratch
+    if (Q.n_q <= direct_max(sc) && !Q.counters) {
         if ((e = launch_direct(db, Q, sc, s)) != cudaSuccess) return e;
         if (n_kernels) *n_kernels = 1;
         return cudaSuccess;

@@ -242,6 +242,14 @@ size_t classify_scratch_bytes(uint32_t n_q_cap, uint32_t sketch_size, uint32_t l
 ClassifyScratch classify_scratch_carve(unsigned char* base, uint32_t n_q_cap, uint32_t sketch_size,
                                        uint32_t large_warps);
 
+// classify_enqueue launches other kernels, and others of their shapes, for
+// few queries than for many, so that one captured launch set does not suit
+// every number of queries up to its capacity: sizes[0 .. n) (ascending, the
+// last is sc's capacity; n is returned) are the numbers of queries up to which
+// a set captured for that number does.
+constexpr int CLASSIFY_MAX_SIZES = 9;
+int classify_set_sizes(const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]);
+
 // Enqueues one launch set (queue reset, lookup + score per chunk, large
 // path) on `s`; no allocation, no synchronisation, so it can be captured
 // in a CUDA graph.  *n_kernels (nullable) receives the kernel launches.
