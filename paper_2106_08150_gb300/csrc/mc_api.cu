@@ -1319,7 +1319,7 @@ int mc_plan_create(const mc_db* db, const mc_classify_params* params, const mc_t
     // the allocations above are stream-ordered on the database stream
     if ((e = cudaStreamSynchronize(db->stream)) != cudaSuccess) return bail(cuda_fail(e, "mc_plan_create"));
     uint32_t sizes[mc::CLASSIFY_MAX_SIZES];
-    p->n_sets = mc::classify_set_sizes(p->sc, sizes);
+    p->n_sets = mc::classify_set_sizes(db_view(db), p->sc, sizes);
     for (int i = 0; i < p->n_sets; ++i) p->sets[i].n_q = sizes[i];
     if ((rc = plan_capture(p, p->sets[p->n_sets - 1]))) return bail(rc);
     *out = p;

@@ -36,7 +36,6 @@ constexpr int WIN_A = 8;                     // windows per query on the shared-
 constexpr uint32_t KB_SLOTS = 1u << 16;      // large-path histogram slots per warp
 constexpr uint32_t LIST_B = MC_MAX_QUERY_WINDOWS * MAX_S;
 constexpr uint32_t LIST_CAP_MAX = WIN_A * MAX_S;  // bucket list of a query of the lookup kernels, any sketch size
-constexpr int B_WARPS_PER_SM = 2;  // large-path CTAs per SM, one piece of global scratch each
 constexpr uint32_t MED_DISTINCT = 1536;      // distinct locations of a query on the medium path
 constexpr int SK_NW = 2;  // windows sketched together
 
@@ -765,6 +764,36 @@ __host__ __device__ constexpr size_t lookup_warp_bytes(uint32_t list_cap) {
     return scratch_bytes<uint16_t>(0, 0, list_cap, BUF_A) + align16(BUF_A + 16) + 2 * STAGED_BYTES;
 }
 
+// Counters of a launch set, behind the large-path queue.  The first two words
+// count over all chunks, those up to QC_WIDEST over one chunk's score
+// kernels; QC_WIDEST belongs to a chunk's lookup.
+enum {
+    QC_LARGE = 0,       // large-path queue length
+    QC_LARGE_WORK = 1,  // its next entry
+    QC_MID = 2,         // medium-path queue length
+    QC_MID_WORK = 3,    // its next entry
+    QC_GROUP = 4,       // next group of sort-path class c: QC_GROUP + c
+    QC_WIDEST = 8,      // most locations of a query, as far as the classes tell them apart
+    QC_END = 9,
+    QC_SAVED = 15       // large-path queue length after the lookup (autotuner)
+};
+
+// The lookup's warps note the size class of their largest query, so that the
+// kernels of classes without a query end at once: handing out groups of
+// queries to find none took each 8 us in launches of 8,000 queries and 20 us
+// from 20,000 on (one counter serves about 10^9 groups/s).  widest holds a
+// number of locations of the highest class that a query is in, or 0 if none
+// is beyond the first.  seen: the warp's own highest so far (a warp writes at
+// most once per class).
+constexpr uint32_t CLASS_0_MAX = 256;
+__device__ __forceinline__ void note_widest(uint32_t* widest, uint32_t locations, uint32_t& seen) {
+    if (locations > max(seen, CLASS_0_MAX)) {
+        atomicMax(widest, locations);
+        // the next class's edge, or no further
+        seen = locations <= 512 ? 512u : (locations <= 1024 ? 1024u : (locations <= 2048 ? 2048u : 0xFFFFFFFFu));
+    }
+}
+
 // Per-query metadata written by the lookup kernel: {found buckets, sliding
 // window size | features << META_FEAT_SHIFT, locations to gather, 32-byte
 // sectors of those locations}, or x = ESCALATED.  On this path a query has
@@ -799,7 +828,7 @@ __global__ void __launch_bounds__(LK_WARPS * 32, 4) k_classify_lookup(ClassifyDb
     const uint32_t nq = min(chunk, total - q0);
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarp = (gridDim.x * blockDim.x) >> 5;
-    uint32_t cur = 0;
+    uint32_t cur = 0, seen = 0;
     if (gw < nq) save_staged(recs, stage_query<true>(db, Q, q0 + gw, buf0, BUF_A, WIN_A));
     for (uint32_t i = gw; i < nq; i += nwarp) {
         cp_async_wait_all();
@@ -828,6 +857,7 @@ __global__ void __launch_bounds__(LK_WARPS * 32, 4) k_classify_lookup(ClassifyDb
             }
         } else if (lane_id() == 0) {
             meta[i] = make_uint4(n_list, sws | (n_feat << META_FEAT_SHIFT), n_locs, n_sect);
+            note_widest(ovf_n + QC_WIDEST, n_locs, seen);
         }
         __syncwarp();
         cur ^= 1;
@@ -879,6 +909,7 @@ struct LookupLanesMem {
     uint32_t q_list[32];       // per query lane: found buckets | features << 16
     uint32_t q_locs[32];       // locations
     uint32_t q_sect[32];       // 32-byte sectors
+    uint32_t seen;             // (note_widest)
     uint16_t inv[LKL_CHUNKS];
 };
 static_assert(LKL_CHUNKS * 16 <= 1u << 13, "staged positions take 13 bits");
@@ -902,6 +933,7 @@ __global__ void __launch_bounds__(LK_WARPS * 32, 3)
     const uint64_t nwarp = (gridDim.x * blockDim.x) >> 5;
     const TableProbe tp(db.fmt);
     const uint32_t lsz = db.jbits ? 4u : 8u;  // bytes per stored location
+    if (lane == 0) M.seen = 0;
 
     for (uint64_t i0 = gw << batch_shift; i0 < nq; i0 += nwarp << batch_shift) {
         // one lane per query: size, status, sliding window
@@ -1183,6 +1215,10 @@ __global__ void __launch_bounds__(LK_WARPS * 32, 3)
             const uint32_t sws = sp >= k ? (sp - k + p.stride - 1) / p.stride + 1 : 0u;
             const uint32_t lf = M.q_list[lane];
             meta[i] = make_uint4(lf & 0xFFFFu, sws | ((lf >> 16) << META_FEAT_SHIFT), M.q_locs[lane], M.q_sect[lane]);
+        }
+        {
+            const uint32_t most = __reduce_max_sync(FULL_MASK, active ? M.q_locs[lane] : 0u);
+            if (lane == 0) note_widest(ovf_n + QC_WIDEST, most, M.seen);
         }
         __syncwarp();
     }
@@ -1882,7 +1918,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     k_classify_sort(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t chunk, uint32_t list_cap,
                     const uint64_t* __restrict__ glist, const uint4* __restrict__ meta, uint32_t h_lo, bool last,
                     uint32_t group_shift, uint32_t* __restrict__ mid_list, uint32_t* __restrict__ mid_n,
-                    uint32_t* __restrict__ group_ctr) {
+                    uint32_t* __restrict__ group_ctr, const uint32_t* __restrict__ widest) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t w = threadIdx.x >> 5;
     const SortMem<E, LocT> M(smem + w * SortMem<E, LocT>::bytes(list_cap), list_cap);
@@ -1890,7 +1926,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     // while this one's last queries finish
     asm volatile("griddepcontrol.launch_dependents;");
     const uint32_t total = total_queries(Q);
-    if (q0 < total) {
+    if (q0 < total && (h_lo == 0 || *widest > h_lo)) {
         ChunkScan it = chunk_scan(min(chunk, total - q0), group_shift, group_ctr);
         uint32_t i;
         uint4 mt;
@@ -1898,7 +1934,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
             const uint64_t* src = glist + (uint64_t)i * list_cap;
             uint32_t distinct;
             bool done = true;
-            if (E == 8 && mt.z <= 32) {
+            if ((E == 8 || (E == 32 && sizeof(LocT) == 8)) && mt.z <= 32) {
                 query_small<LocT>(db, Q, q0 + i, src, mt.x, meta_sws(mt), mt.z, distinct);
             } else {
                 sort_gather<E>(db, M, src, mt.x, mt.z);
@@ -1946,16 +1982,19 @@ constexpr uint32_t BLK_LIST = MC_MAX_QUERY_WINDOWS * MAX_S;  // buckets of one q
 constexpr uint32_t BLK_CNT = 4096;                           // block counters
 constexpr uint32_t BLK_HASH = 4096;                          // slots of the distinct survivors,
 constexpr uint32_t BLK_DISTINCT = 2048;                      // of which as many are used (what a warp sorts)
+constexpr int BLK_CTAS = 2;                                  // resident per SM
 constexpr int BLK_STEP = 8;                                  // consecutive locations per thread and step
 
 template <class LocT>
 struct BlockMem {
     uint64_t list[BLK_LIST];      // found buckets, offset << 16 | size
     uint32_t pre[BLK_LIST + 4];   // exclusive prefix of their sizes
-    uint32_t cnt[BLK_CNT];
-    LocT key[BLK_HASH];           // distinct surviving locations, hashed,
+    union {
+        uint32_t cnt[BLK_CNT];    // block counters, until the survivors are chosen
+        LocT loc[BLK_DISTINCT];   // the distinct survivors, sorted
+    };
+    LocT key[BLK_HASH];           // the distinct survivors, hashed,
     uint32_t times[BLK_HASH];     // and how often each was gathered
-    LocT loc[BLK_DISTINCT + 4];   // the same sorted
     uint32_t rs[BLK_DISTINCT + 4];
     union {
         uint32_t score[BLK_DISTINCT + 4];
@@ -1969,6 +2008,8 @@ struct BlockMem {
     uint32_t n_list, sect, n, T, n_win, sws, n_feat, work;
     int status;
 };
+
+static_assert(BLK_CTAS * (sizeof(BlockMem<uint64_t>) + 1024) <= 228 * 1024, "shared memory of an SM");
 
 // f(location) for every location of the query's n_list buckets (H in all).
 template <class LocT, class F>
@@ -1995,6 +2036,17 @@ __device__ __forceinline__ void block_for_each(const ClassifyDb& db, const Block
         for (int u = 0; u < BLK_STEP; ++u)
             if (x0 + u < H) f(v[u]);
     }
+}
+
+// The block counters once more, for a query that is done again (out of line:
+// one in thousands).  Between barriers, ends with one.
+template <class LocT>
+__device__ __noinline__ void block_count_again(const ClassifyDb& db, BlockMem<LocT>& B, uint32_t n_list, uint32_t H,
+                                               const BlockSlot<LocT>& bs) {
+    for (uint32_t i = threadIdx.x; i < BLK_CNT; i += BLK_THREADS) B.cnt[i] = 0;
+    __syncthreads();
+    block_for_each(db, B, n_list, H, [&](LocT x) { atomicAdd(&B.cnt[bs(x, BLK_CNT - 1)], 1u); });
+    __syncthreads();
 }
 
 // Steps 5-8 of the query whose n_list buckets are in B.list, by the whole
@@ -2110,6 +2162,7 @@ __device__ __forceinline__ bool block_score(const ClassifyDb& db, const Classify
         T = B.T;
         distinct = D;
         if (T == 0) return true;
+        if (T > 1) block_count_again<LocT>(db, B, n_list, H, bs);  // (the survivors took the counters' place)
     }
 }
 
@@ -2118,7 +2171,7 @@ __device__ __forceinline__ bool block_score(const ClassifyDb& db, const Classify
 // over from the lookup; queries of more than MED_DISTINCT distinct locations
 // go to the large path.
 template <class LocT>
-__global__ void __launch_bounds__(BLK_THREADS, 2) k_classify_medium(ClassifyDb db, ClassifyQuery Q, uint32_t q0,
+__global__ void __launch_bounds__(BLK_THREADS, BLK_CTAS) k_classify_medium(ClassifyDb db, ClassifyQuery Q, uint32_t q0,
                                                                    uint32_t list_cap,
                                                                    const uint64_t* __restrict__ glist,
                                                                    const uint4* __restrict__ meta,
@@ -2256,7 +2309,7 @@ __device__ __forceinline__ void block_lookup(const ClassifyDb& db, const Classif
 // fit the CTA's memory is processed by one warp with working memory in
 // global scratch (one piece per CTA).
 template <int R, int KC, class LocT>
-__global__ void __launch_bounds__(BLK_THREADS, 2) k_classify_large(ClassifyDb db, ClassifyQuery Q,
+__global__ void __launch_bounds__(BLK_THREADS, BLK_CTAS) k_classify_large(ClassifyDb db, ClassifyQuery Q,
                                                                    const uint32_t* __restrict__ ovf_list,
                                                                    const uint32_t* __restrict__ ovf_n,
                                                                    uint32_t* __restrict__ work,
@@ -2397,12 +2450,13 @@ LargeKernel pick_large(const ClassifyDb& db) {
 
 // Kernels and launch shapes of one launch set.
 using SortKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint32_t, const uint64_t*, const uint4*,
-                            uint32_t, bool, uint32_t, uint32_t*, uint32_t*, uint32_t*);
+                            uint32_t, bool, uint32_t, uint32_t*, uint32_t*, uint32_t*, const uint32_t*);
 
 // The sort path's size classes: queries of up to 256, 512, 1024 and 2048
 // gathered locations, each with its own kernel (E = 8, 16, 32, 64 per lane).
 constexpr int N_SORT_CLASSES = 4;
-constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {256, 512, 1024, 2048};
+constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {CLASS_0_MAX, 512, 1024, 2048};
+static_assert(QC_WIDEST - QC_GROUP == N_SORT_CLASSES, "a group counter per class");
 
 // Launches of at least this many queries look up with one window per lane:
 // four to five for each of the 3,648 resident warps; with fewer, lanes stay
@@ -2411,6 +2465,15 @@ constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {256, 512, 1024, 2048};
 // 168 / 68; half pairs, lengths 50-300, 8,000 queries 38 / 39, 20,000 73 / 65,
 // 100,000 276 / 180.
 constexpr uint32_t LANES_MIN_QUERIES = 16384;
+
+// Launches of at most this many queries for each resident warp of the largest
+// sort class leave them all to that class, with 64-bit locations: its warps
+// have the room, and the other classes' kernels, of 2 us each with nothing to
+// do, are not launched (1,000 pairs of 100, draft assemblies: 34.5 us, here 32.4).
+// With 32-bit locations the largest class runs before the medium path and the
+// others beside it, which is worth more where that path has queries (1,000
+// pairs, repeat-rich genomes: 122 us, 129 in one class).
+constexpr uint32_t ONE_CLASS_ROUNDS = 2;
 
 struct Geometry {
     LookupKernel kl;         // one window per warp
@@ -2422,6 +2485,7 @@ struct Geometry {
     SortKernel kt[N_SORT_CLASSES];
     bool sort;           // score by the sort path (else the hash path)
     int n_sort;          // sort classes in use
+    bool one_class;      // the largest takes them all
     uint32_t list_cap;
     size_t smem_l, smem_s, smem_m, smem_b, per_warp_b, smem_t[N_SORT_CLASSES];
     uint32_t threads_l, threads_s, grid_l, grid_s, grid_m, blocks_b, grid_t[N_SORT_CLASSES];
@@ -2455,7 +2519,10 @@ cudaError_t resident_ctas(const void* kernel, uint32_t threads, size_t smem, int
     return e;
 }
 
-cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratch& sc, Geometry* g) {
+// counting: a call with counters, which drops no location before the sort;
+// then 64-bit locations, of which no class sorts more than 256, take the hash
+// path.
+cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratch& sc, bool counting, Geometry* g) {
     cudaError_t e;
     int dev = 0, sms = NUM_SMS_HINT;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -2474,7 +2541,7 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->smem_m = blk;
     if ((e = allow_smem(g->km, g->smem_m)) != cudaSuccess) return e;
     if ((e = allow_smem(g->kb, g->smem_b)) != cudaSuccess) return e;
-    g->grid_m = std::min<uint32_t>((uint32_t)sms * 2, std::max<uint32_t>(sc.chunk, 1));
+    g->grid_m = std::min<uint32_t>((uint32_t)sms * BLK_CTAS, std::max<uint32_t>(sc.chunk, 1));
     g->threads_l = t.lookup_warps * 32;
     g->threads_s = t.score_warps * 32;
     const auto lookup_bytes = [&](uint32_t lc) { return g->kll ? sizeof(LookupLanesMem) : lookup_warp_bytes(lc); };
@@ -2509,8 +2576,9 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->per_warp_b = scratch_bytes<uint32_t>(KB_SLOTS, LIST_B, LIST_B, BUF_B);
     g->blocks_b = std::max<uint32_t>(1, std::min(sc.large_warps, sc.n_q_cap));  // one piece of global scratch each
     // sort path: locations sorted as they are stored (not with wide keys of 32-bit ones)
-    g->sort = km != KeyMode::wide32 && t.score_mode != SCORE_HASH;
+    g->sort = km != KeyMode::wide32 && t.score_mode != SCORE_HASH && !(counting && km == KeyMode::wide64);
     g->n_sort = 0;
+    g->one_class = false;
     g->group_shift = 0;
     if (g->sort) {
         const SortKernel kts[N_SORT_CLASSES] = {
@@ -2543,6 +2611,8 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
                                                          (uint64_t)sms * std::max(occ_t, 1));
             g->n_sort = c2 + 1;
         }
+        const uint64_t last_warps = (uint64_t)g->grid_t[g->n_sort - 1] * SORT_WARPS;
+        g->one_class = !compact && !counting && c <= ONE_CLASS_ROUNDS * last_warps;
     }
     return cudaSuccess;
 }
@@ -2570,10 +2640,6 @@ constexpr ScratchLayout scratch_layout(uint32_t n_q_cap, uint32_t sketch_size, u
     return L;
 }
 
-// Queue counters: [0] large-path queue length, [1] large-path work counter,
-// [2] medium-path queue length, [3] medium-path work counter, [4] saved
-// large-path queue length (autotuner), [5 + c] group counter of sort-path
-// class c.
 uint32_t* queue_counters(const ClassifyScratch& sc) { return sc.ovf + sc.n_q_cap; }
 
 cudaError_t launch_lookup(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
@@ -2594,21 +2660,26 @@ cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const Classif
                           uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
     MC_LAUNCH("classify_medium", s,
-              g.km<<<g.grid_m, BLK_THREADS, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid, qc + 2,
-                                                             qc + 3, sc.ovf, qc));
+              g.km<<<g.grid_m, BLK_THREADS, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid,
+                                                         qc + QC_MID, qc + QC_MID_WORK, sc.ovf, qc + QC_LARGE));
     return cudaGetLastError();
 }
 
 // A launch of few queries: all of them straight to the large path's kernel.
-// One launch instead of the six kernels and three memsets of a launch set,
+// One launch instead of the six kernels and a memset of a launch set,
 // whose latency is what such a call takes: 16 pairs 25 us on the device
 // against 65.  One wave of CTAs (two per SM) holds 304 queries; 2,000 take
 // 115 us this way and 61 the other (reads of 100), so the line lies between.
+// With 64-bit locations a launch set is shorter (one size class), and the line
+// is one wave: pairs of 100, draft assemblies, 200 queries 23 us this way and
+// 30 the other, 400 queries 38 and 31 (54 and 37 with candidate lists).
 constexpr uint32_t DIRECT_MAX_QUERIES = 512;
 
-// (a CTA per piece of global scratch, and at most two queries each: of an
-// allocation-free launch, which has eight, 16 queries)
-uint32_t direct_max(const ClassifyScratch& sc) { return std::min(DIRECT_MAX_QUERIES, 2 * sc.large_warps); }
+// (a CTA per piece of global scratch, and at most two queries each, or one
+// with 64-bit locations: an allocation-free launch has eight)
+uint32_t direct_max(const ClassifyDb& db, const ClassifyScratch& sc) {
+    return std::min(DIRECT_MAX_QUERIES, (db.jbits ? 2 : 1) * sc.large_warps);
+}
 
 cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc, cudaStream_t s) {
     const LargeKernel kb = pick_large(db);
@@ -2622,7 +2693,13 @@ cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const Cl
     return cudaGetLastError();
 }
 
-// Score of the chunk at q0.  Sort path, 32-bit locations: the largest size
+// Zeroes the counters from..to of a launch set.
+cudaError_t reset_counters(const ClassifyScratch& sc, int from, int to, cudaStream_t s) {
+    return cudaMemsetAsync(queue_counters(sc) + from, 0, (to - from) * sizeof(uint32_t), s);
+}
+
+// Score of the chunk at q0, whose counters QC_MID .. QC_WIDEST are zero (each
+// launch appends up to a chunk's queries to the queues).  Sort path, 32-bit locations: the largest size
 // class first (it queues the queries beyond it), then the medium path, then
 // the other classes, the most populous one (512) first.  Each of those is
 // launched with programmatic stream serialization, so that it fills the SMs
@@ -2635,13 +2712,11 @@ cudaError_t launch_direct(const ClassifyDb& db, const ClassifyQuery& Q, const Cl
 cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
                          uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
-    cudaError_t e = cudaMemsetAsync(qc + 2, 0, 2 * sizeof(uint32_t), s);  // medium queue; [4] is kept
-    if (e != cudaSuccess) return e;
-    if (g.sort && (e = cudaMemsetAsync(qc + 5, 0, N_SORT_CLASSES * sizeof(uint32_t), s)) != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (!g.sort) {
         MC_LAUNCH("classify_score", s,
                   g.ks<<<g.grid_s, g.threads_s, g.smem_s, s>>>(db, Q, q0, sc.chunk, g.list_cap, sc.glist, sc.meta,
-                                                              sc.mid, qc + 2));
+                                                              sc.mid, qc + QC_MID));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         return launch_medium(g, db, Q, sc, q0, s);
     }
@@ -2652,8 +2727,8 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
     int order[N_SORT_CLASSES + 1], n = 0;
     order[n++] = last;
     if (narrow) order[n++] = -1;  // medium path
-    if (last >= 2) order[n++] = 1;
-    for (int c = 0; c < last; ++c)
+    if (last >= 2 && !g.one_class) order[n++] = 1;
+    for (int c = 0; c < last && !g.one_class; ++c)
         if (c != 1 || last < 2) order[n++] = c;
     if (!narrow) order[n++] = -1;
     for (int k = 0; k < n; ++k) {
@@ -2662,7 +2737,7 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
             if ((e = launch_medium(g, db, Q, sc, q0, s)) != cudaSuccess) return e;
             continue;
         }
-        const uint32_t h_lo = c ? SORT_CLASS_MAX[c - 1] : 0;
+        const uint32_t h_lo = c && !g.one_class ? SORT_CLASS_MAX[c - 1] : 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(g.grid_t[c]);
         cfg.blockDim = dim3(SORT_WARPS * 32);
@@ -2676,7 +2751,8 @@ cudaError_t launch_score(const Geometry& g, const ClassifyDb& db, const Classify
         MC_LAUNCH(names[c], s,
                   e = cudaLaunchKernelEx(&cfg, g.kt[c], db, Q, q0, (uint32_t)sc.chunk, g.list_cap,
                                          (const uint64_t*)sc.glist, (const uint4*)sc.meta, h_lo, c == last, g.group_shift,
-                                         sc.mid, qc + 2, qc + 5 + c));
+                                         sc.mid, qc + QC_MID, qc + QC_GROUP + c,
+                                         (const uint32_t*)qc + QC_WIDEST));
         if (e != cudaSuccess) return e;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -2687,7 +2763,8 @@ cudaError_t launch_large(const Geometry& g, const ClassifyDb& db, const Classify
                          cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
     MC_LAUNCH("classify_large", s,
-              g.kb<<<g.blocks_b, BLK_THREADS, g.smem_b, s>>>(db, Q, sc.ovf, qc, qc + 1, sc.large, g.per_warp_b));
+              g.kb<<<g.blocks_b, BLK_THREADS, g.smem_b, s>>>(db, Q, sc.ovf, qc + QC_LARGE, qc + QC_LARGE_WORK, sc.large,
+                                                        g.per_warp_b));
     return cudaGetLastError();
 }
 
@@ -2813,7 +2890,7 @@ uint32_t classify_default_large_warps() {
         cudaGetLastError();
         sms = NUM_SMS_HINT;
     }
-    return (uint32_t)(sms * B_WARPS_PER_SM);
+    return (uint32_t)(sms * BLK_CTAS);
 }
 
 size_t classify_scratch_bytes(uint32_t n_q_cap, uint32_t sketch_size, uint32_t large_warps) {
@@ -2835,12 +2912,12 @@ ClassifyScratch classify_scratch_carve(unsigned char* base, uint32_t n_q_cap, ui
     return sc;
 }
 
-int classify_set_sizes(const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]) {
+int classify_set_sizes(const ClassifyDb& db, const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]) {
     int n = 0;
     const auto add = [&](uint32_t most) {
         if (most < sc.n_q_cap) sizes[n++] = most;
     };
-    add(direct_max(sc));
+    add(direct_max(db, sc));
     add(LANES_MIN_QUERIES - 1);
     // from there on shapes change every doubling: the lookup's queries per warp
     // at 8 and 16 times its 3,648 resident warps (the sizes lie just under
@@ -2859,19 +2936,19 @@ cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const
     if (Q.n_q > scratch.n_q_cap) return cudaErrorInvalidValue;
     ClassifyScratch sc = scratch;
     sc.chunk = std::min(sc.chunk, Q.n_q);  // the launch's shape follows its queries, not its scratch
-    if (Q.n_q <= direct_max(sc) && !Q.counters) {
+    if (Q.n_q <= direct_max(db, sc) && !Q.counters) {
         if ((e = launch_direct(db, Q, sc, s)) != cudaSuccess) return e;
         if (n_kernels) *n_kernels = 1;
         return cudaSuccess;
     }
     Geometry g;
-    if ((e = geometry(db, t, sc, &g)) != cudaSuccess) return e;
-    // only the queue counters must start at zero
-    if ((e = cudaMemsetAsync(queue_counters(sc), 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return e;
+    if ((e = geometry(db, t, sc, Q.counters != nullptr, &g)) != cudaSuccess) return e;
     for (uint32_t q0 = 0; q0 < Q.n_q; q0 += sc.chunk) {
+        // only the counters must start at zero
+        if ((e = reset_counters(sc, q0 ? QC_MID : QC_LARGE, QC_END, s)) != cudaSuccess) return e;
         if ((e = launch_lookup(g, db, Q, sc, q0, s)) != cudaSuccess) return e;
         if ((e = launch_score(g, db, Q, sc, q0, s)) != cudaSuccess) return e;
-        n += 2 + (g.sort ? g.n_sort : 1);
+        n += 2 + (g.sort && !g.one_class ? g.n_sort : 1);
         if (sc.chunk == 0) break;
     }
     if ((e = launch_large(g, db, Q, sc, s)) != cudaSuccess) return e;
@@ -2947,11 +3024,11 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
                 t.probe_batch = lb;
                 t.lookup_warps = lw;
                 Geometry g;
-                if ((e = geometry(db, t, sc, &g)) != cudaSuccess) goto done;
+                if ((e = geometry(db, t, sc, Q.counters != nullptr, &g)) != cudaSuccess) goto done;
                 float ms = 0;
                 e = timed(
                     [&]() -> cudaError_t {
-                        cudaError_t err = cudaMemsetAsync(qc, 0, 2 * sizeof(uint32_t), s);
+                        cudaError_t err = reset_counters(sc, QC_LARGE, QC_END, s);
                         return err != cudaSuccess ? err : launch_lookup(g, db, Q, sc, 0, s);
                     },
                     &ms);
@@ -2969,13 +3046,25 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
     // lookup output of the chosen setting, and its queue length, for stage 1
     {
         Geometry g;
-        if ((e = geometry(db, cur, sc, &g)) != cudaSuccess) goto done;
-        if ((e = cudaMemsetAsync(qc, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) goto done;
+        if ((e = geometry(db, cur, sc, Q.counters != nullptr, &g)) != cudaSuccess) goto done;
+        if ((e = reset_counters(sc, QC_LARGE, QC_END, s)) != cudaSuccess) goto done;
         if ((e = launch_lookup(g, db, Q, sc, 0, s)) != cudaSuccess) goto done;
-        if ((e = cudaMemcpyAsync(qc + 4, qc, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) != cudaSuccess) goto done;
+        if ((e = cudaMemcpyAsync(qc + QC_SAVED, qc + QC_LARGE, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) !=
+            cudaSuccess)
+            goto done;
     }
-    // stage 1: score settings (with the large path they leave)
+    // stage 1: score settings (with the large path they leave), each from the
+    // lookup's output and its counters as the lookup left them
     {
+        const auto score_again = [&](const Geometry& g) -> cudaError_t {
+            cudaError_t err;
+            if ((err = cudaMemcpyAsync(qc + QC_LARGE, qc + QC_SAVED, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) !=
+                cudaSuccess)
+                return err;
+            if ((err = reset_counters(sc, QC_LARGE_WORK, QC_WIDEST, s)) != cudaSuccess) return err;
+            if ((err = launch_score(g, db, Q, sc, 0, s)) != cudaSuccess) return err;
+            return launch_large(g, db, Q, sc, s);
+        };
         bool first = true;
         Tuning bs = cur;
         for (uint32_t ka : {256u, 512u, 1024u}) {
@@ -2987,19 +3076,9 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
                     t.gather_batch = gb;
                     t.score_warps = sw;
                     Geometry g;
-                    if ((e = geometry(db, t, sc, &g)) != cudaSuccess) goto done;
+                    if ((e = geometry(db, t, sc, Q.counters != nullptr, &g)) != cudaSuccess) goto done;
                     float ms = 0;
-                    e = timed(
-                        [&]() -> cudaError_t {
-                            cudaError_t err;
-                            if ((err = cudaMemcpyAsync(qc, qc + 4, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) !=
-                                cudaSuccess)
-                                return err;
-                            if ((err = cudaMemsetAsync(qc + 1, 0, sizeof(uint32_t), s)) != cudaSuccess) return err;
-                            if ((err = launch_score(g, db, Q, sc, 0, s)) != cudaSuccess) return err;
-                            return launch_large(g, db, Q, sc, s);
-                        },
-                        &ms);
+                    e = timed([&]() -> cudaError_t { return score_again(g); }, &ms);
                     if (e != cudaSuccess) goto done;
                     if (records) records->push_back(TuneRecord{t, 1, ms});
                     if (first || ms < best_ms) {
@@ -3018,19 +3097,9 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
                 t.sort_max = smax;
                 t.wide_keys = 0;
                 Geometry g;
-                if ((e = geometry(db, t, sc, &g)) != cudaSuccess) goto done;
+                if ((e = geometry(db, t, sc, Q.counters != nullptr, &g)) != cudaSuccess) goto done;
                 float ms = 0;
-                e = timed(
-                    [&]() -> cudaError_t {
-                        cudaError_t err;
-                        if ((err = cudaMemcpyAsync(qc, qc + 4, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) !=
-                            cudaSuccess)
-                            return err;
-                        if ((err = cudaMemsetAsync(qc + 1, 0, sizeof(uint32_t), s)) != cudaSuccess) return err;
-                        if ((err = launch_score(g, db, Q, sc, 0, s)) != cudaSuccess) return err;
-                        return launch_large(g, db, Q, sc, s);
-                    },
-                    &ms);
+                e = timed([&]() -> cudaError_t { return score_again(g); }, &ms);
                 if (e != cudaSuccess) goto done;
                 if (records) records->push_back(TuneRecord{t, 1, ms});
                 if (ms < best_ms) {

@@ -248,7 +248,7 @@ ClassifyScratch classify_scratch_carve(unsigned char* base, uint32_t n_q_cap, ui
 // last is sc's capacity; n is returned) are the numbers of queries up to which
 // a set captured for that number does.
 constexpr int CLASSIFY_MAX_SIZES = 9;
-int classify_set_sizes(const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]);
+int classify_set_sizes(const ClassifyDb& db, const ClassifyScratch& sc, uint32_t sizes[CLASSIFY_MAX_SIZES]);
 
 // Enqueues one launch set (queue reset, lookup + score per chunk, large
 // path) on `s`; no allocation, no synchronisation, so it can be captured
