@@ -773,8 +773,10 @@ enum {
     QC_MID = 2,         // medium-path queue length
     QC_MID_WORK = 3,    // its next entry
     QC_GROUP = 4,       // next group of sort-path class c: QC_GROUP + c
-    QC_WIDEST = 8,      // most locations of a query, as far as the classes tell them apart
-    QC_END = 9,
+    QC_QUEUED_WORK = 8, // next entry of the queue that warps take
+    QC_REST = 9,        // length of the queue of what they leave
+    QC_WIDEST = 10,     // most locations of a query, as far as the classes tell them apart
+    QC_END = 11,
     QC_SAVED = 15       // large-path queue length after the lookup (autotuner)
 };
 
@@ -1450,6 +1452,7 @@ __device__ __forceinline__ void warp_bitonic_sort(T (&k)[E]) {
 constexpr int SORT_WARPS = 4;           // warps per CTA of the sort path
 constexpr int GU = 4;                   // gather steps unrolled together
 constexpr uint32_t SMALL_SORT = 256;    // survivors that are sorted eight per lane
+constexpr uint32_t QUEUED_MAX = 1024;   // locations of a queued query that a warp sorts
 constexpr uint32_t NO_FILTER = 64;      // locations that are sorted without a look at the counts
 
 // Per-warp shared memory of the sort path: the buckets' location indices,
@@ -1964,6 +1967,54 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Queries that the hash path's score kernel or a small sort_max leaves, as
+// far as a warp can sort them: up to 1,024 locations, a warp each, off the
+// queue mid_list; the rest go on to the medium path's CTAs (rest_list).
+// There are many of them where the tuning draws the line low, and a CTA for
+// each is slow (200,000 mixed reads, 1,000 genomes, sort_max 256: 4.66 ms, here
+// 0.98; score_mode 2 with 256 slots: 4.87 ms, here 1.22).  Lines of 1,024 leave
+// few that a warp could take, and the kernel is not launched.
+template <class LocT>
+__global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<32, LocT>())
+    k_sort_queued(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t list_cap, const uint64_t* __restrict__ glist,
+                  const uint4* __restrict__ meta, const uint32_t* __restrict__ mid_list,
+                  const uint32_t* __restrict__ mid_n, uint32_t* __restrict__ work, uint32_t* __restrict__ rest_list,
+                  uint32_t* __restrict__ rest_n) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t lane = lane_id();
+    const SortMem<32, LocT> M(smem + (threadIdx.x >> 5) * SortMem<32, LocT>::bytes(list_cap), list_cap);
+    const uint32_t n = *mid_n;
+    for (;;) {
+        uint32_t k = 0;
+        if (lane == 0) k = atomicAdd(work, 1u);
+        k = __shfl_sync(FULL_MASK, k, 0);
+        if (k >= n) break;
+        const uint32_t i = mid_list[k];
+        const uint4 mt = meta[i];
+        uint32_t distinct = 0;
+        bool done = false;
+        if (mt.z <= QUEUED_MAX) {
+            sort_gather<32>(db, M, glist + (uint64_t)i * list_cap, mt.x, mt.z);
+            cp_async_wait_all();
+            __syncwarp();
+            done = query_sort<32>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct);
+        }
+        if (!done) {
+            if (lane == 0) rest_list[atomicAdd(rest_n, 1u)] = i;
+        } else if (Q.counters) {
+            Counters ctr;
+            ctr.features = meta_feat(mt);
+            ctr.locations = mt.z;
+            ctr.distinct = distinct;
+            ctr.found = mt.x;
+            ctr.sectors = mt.w;
+            ctr.queries = 1;
+            flush_counters(Q, ctr, KC_MEDIUM);
+            if (lane == 0) atomicAdd(Q.counters + 6, 1ull);
+        }
+    }
+}
+
 // ------------------------------------------------------------------
 // Queries beyond the sort path's size classes: one CTA per query.  All its
 // threads gather, count by block and drop locations as in query_sort, with
@@ -2357,6 +2408,9 @@ __global__ void __launch_bounds__(BLK_THREADS, BLK_CTAS) k_classify_large(Classi
 
 constexpr uint32_t CHUNK = CLASSIFY_CHUNK;
 
+using QueuedKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, const uint64_t*, const uint4*,
+                              const uint32_t*, const uint32_t*, uint32_t*, uint32_t*, uint32_t*);
+
 using LookupKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint32_t, uint64_t*, uint4*, uint32_t*,
                               uint32_t*);
 using ScoreKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint32_t, const uint64_t*, const uint4*,
@@ -2456,7 +2510,7 @@ using SortKernel = void (*)(ClassifyDb, ClassifyQuery, uint32_t, uint32_t, uint3
 // gathered locations, each with its own kernel (E = 8, 16, 32, 64 per lane).
 constexpr int N_SORT_CLASSES = 4;
 constexpr uint32_t SORT_CLASS_MAX[N_SORT_CLASSES] = {CLASS_0_MAX, 512, 1024, 2048};
-static_assert(QC_WIDEST - QC_GROUP == N_SORT_CLASSES, "a group counter per class");
+static_assert(QC_QUEUED_WORK - QC_GROUP == N_SORT_CLASSES, "a group counter per class");
 
 // Launches of at least this many queries look up with one window per lane:
 // four to five for each of the 3,648 resident warps; with fewer, lanes stay
@@ -2481,14 +2535,15 @@ struct Geometry {
     uint32_t batch_shift;    // log2 of the queries a lookup warp takes at a time (kll)
     ScoreKernel ks;
     MediumKernel km;
+    QueuedKernel kq;  // queued queries of up to QUEUED_MAX locations, or nullptr
     LargeKernel kb;
     SortKernel kt[N_SORT_CLASSES];
     bool sort;           // score by the sort path (else the hash path)
     int n_sort;          // sort classes in use
     bool one_class;      // the largest takes them all
     uint32_t list_cap;
-    size_t smem_l, smem_s, smem_m, smem_b, per_warp_b, smem_t[N_SORT_CLASSES];
-    uint32_t threads_l, threads_s, grid_l, grid_s, grid_m, blocks_b, grid_t[N_SORT_CLASSES];
+    size_t smem_l, smem_s, smem_m, smem_b, smem_q, per_warp_b, smem_t[N_SORT_CLASSES];
+    uint32_t threads_l, threads_s, grid_l, grid_s, grid_m, grid_q, blocks_b, grid_t[N_SORT_CLASSES];
     uint32_t group_shift;  // log2 of the queries a sort-path warp takes at a time
 };
 
@@ -2614,13 +2669,27 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
         const uint64_t last_warps = (uint64_t)g->grid_t[g->n_sort - 1] * SORT_WARPS;
         g->one_class = !compact && !counting && c <= ONE_CLASS_ROUNDS * last_warps;
     }
+    g->kq = nullptr;
+    // (queries beyond this many locations are queued)
+    const uint32_t line = g->sort ? SORT_CLASS_MAX[g->n_sort - 1] : t.hist_slots;
+    if (line < QUEUED_MAX) {
+        const auto bytes = [&](uint32_t lc) {
+            return SORT_WARPS * (db.jbits ? SortMem<32, uint32_t>::bytes(lc) : SortMem<32, uint64_t>::bytes(lc));
+        };
+        g->kq = db.jbits ? k_sort_queued<uint32_t> : k_sort_queued<uint64_t>;
+        g->smem_q = bytes(g->list_cap);
+        if ((e = allow_smem(g->kq, bytes(LIST_CAP_MAX))) != cudaSuccess) return e;
+        int occ_q = 1;
+        if ((e = resident_ctas((const void*)g->kq, SORT_WARPS * 32, g->smem_q, dev, &occ_q)) != cudaSuccess) return e;
+        g->grid_q = (uint32_t)std::min<uint64_t>((c + SORT_WARPS - 1) / SORT_WARPS, (uint64_t)sms * std::max(occ_q, 1));
+    }
     return cudaSuccess;
 }
 
 __host__ __device__ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scratch layout: escalation queue + counters, chunk metadata, medium-path
-// queue, chunk bucket lists, large-path working memory.
+// queue and the queue of what warps leave of it, chunk bucket lists, large-path working memory.
 struct ScratchLayout {
     size_t ovf, meta, mid, glist, large, total;
     uint32_t chunk;
@@ -2634,7 +2703,7 @@ constexpr ScratchLayout scratch_layout(uint32_t n_q_cap, uint32_t sketch_size, u
     L.ovf = 0;
     L.meta = align256(L.ovf + ((size_t)n_q_cap + 16) * 4);
     L.mid = align256(L.meta + (size_t)L.chunk * sizeof(uint4));
-    L.glist = align256(L.mid + (size_t)L.chunk * 4);
+    L.glist = align256(L.mid + (size_t)L.chunk * 4 * 2);
     L.large = align256(L.glist + (size_t)L.chunk * list_cap * 8);
     L.total = align256(L.large + (size_t)large_warps * per_warp_b);
     return L;
@@ -2659,9 +2728,22 @@ cudaError_t launch_lookup(const Geometry& g, const ClassifyDb& db, const Classif
 cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const ClassifyQuery& Q, const ClassifyScratch& sc,
                           uint32_t q0, cudaStream_t s) {
     uint32_t* qc = queue_counters(sc);
+    const uint32_t* queue = sc.mid;
+    uint32_t* queue_n = qc + QC_MID;
+    if (g.kq) {
+        uint32_t* rest = sc.mid + sc.chunk;
+        MC_LAUNCH("classify_queued", s,
+                  g.kq<<<g.grid_q, SORT_WARPS * 32, g.smem_q, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid,
+                                                                 qc + QC_MID, qc + QC_QUEUED_WORK, rest,
+                                                                 qc + QC_REST));
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        queue = rest;
+        queue_n = qc + QC_REST;
+    }
     MC_LAUNCH("classify_medium", s,
-              g.km<<<g.grid_m, BLK_THREADS, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, sc.mid,
-                                                         qc + QC_MID, qc + QC_MID_WORK, sc.ovf, qc + QC_LARGE));
+              g.km<<<g.grid_m, BLK_THREADS, g.smem_m, s>>>(db, Q, q0, g.list_cap, sc.glist, sc.meta, queue, queue_n,
+                                                         qc + QC_MID_WORK, sc.ovf, qc + QC_LARGE));
     return cudaGetLastError();
 }
 
@@ -2948,7 +3030,7 @@ cudaError_t classify_enqueue(const ClassifyDb& db, const ClassifyQuery& Q, const
         if ((e = reset_counters(sc, q0 ? QC_MID : QC_LARGE, QC_END, s)) != cudaSuccess) return e;
         if ((e = launch_lookup(g, db, Q, sc, q0, s)) != cudaSuccess) return e;
         if ((e = launch_score(g, db, Q, sc, q0, s)) != cudaSuccess) return e;
-        n += 2 + (g.sort && !g.one_class ? g.n_sort : 1);
+        n += 2 + (g.sort && !g.one_class ? g.n_sort : 1) + (g.kq ? 1 : 0);
         if (sc.chunk == 0) break;
     }
     if ((e = launch_large(g, db, Q, sc, s)) != cudaSuccess) return e;

@@ -232,7 +232,7 @@ bool tuning_valid(const Tuning& t);
 struct ClassifyScratch {
     uint32_t* ovf;         // large-path queue (n_q_cap) + queue counters
     uint4* meta;           // per query of a chunk
-    uint32_t* mid;         // medium-path queue of a chunk
+    uint32_t* mid;         // medium-path queues of a chunk (two)
     uint64_t* glist;       // bucket lists of a chunk
     unsigned char* large;  // large-path working memory: large_warps pieces, one per CTA
     uint32_t n_q_cap, chunk, large_warps;
