@@ -181,9 +181,10 @@ constexpr uint32_t WINDOWS_PER_TASK = 16;
 constexpr int SK_NW = 2;  // windows sketched together by a warp
 
 // One warp per window (sketch sizes above 16, which lane_sketch does not
-// take); a warp takes WINDOWS_PER_TASK consecutive windows and walks the
-// sequences they belong to.  EMIT = build pairs, else the
-// debug sketch export.  Five resident blocks per SM (48 registers).
+// take, and k-mers so short that they repeat); a warp takes
+// WINDOWS_PER_TASK consecutive windows and walks the sequences they belong
+// to.  EMIT = build pairs, else the debug sketch export.  Five resident
+// blocks per SM (48 registers).
 template <int R, int KC, bool EMIT>
 __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq, const uint8_t* __restrict__ seq,
                                                const uint64_t* __restrict__ offs,
@@ -258,12 +259,15 @@ __global__ void __launch_bounds__(BT, 5) k_sketch(SketchParams p, uint32_t n_seq
 // Windows of consecutive targets are in memory order too; should targets too
 // short for a window lie between them and spread the 32 windows over more
 // bytes than the staging area holds, the windows that fit are taken first.
-// A window that lane_sketch does not settle is sketched by the whole warp.
+// A window that lane_sketch does not settle is sketched by the whole warp, and
+// where more than EMIT_LANE_EXACT of the 32 are left, those by their lanes
+// (lane_sketch_exact).
 // Bound by the integer ALU (74-80% busy, half the issue rate; 118 warp
 // instructions per window): 14.3 Gbp of the large workload take 20.5 ms (127 M
 // windows of 113 k-mers), against 64.5 ms with one warp per window.  Six CTAs
 // per SM: 5% and 15% faster than five and four.
 constexpr uint32_t EMIT_CAP = 48;  // candidates per lane
+constexpr int EMIT_LANE_EXACT = 12;  // (by their lanes, 32 cost what 8 to 17 do one by one)
 __host__ __device__ constexpr uint32_t emit_stage_words(const SketchParams& p) {
     return (31 * p.stride + p.w + 30) / 16 + 2;
 }
@@ -364,6 +368,13 @@ __global__ void __launch_bounds__(EMIT_WARPS * 32, EMIT_CTAS)
                 uint32_t* feat = cand;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) feat[i * LS_FEAT_STRIDE + lane] = v[i];
+                if (__popc(again) > EMIT_LANE_EXACT) {
+                    const bool mine = (again >> lane) & 1u;
+                    const uint32_t c = lane_sketch_exact<KC>(code, inv, n_ch, in ? (uint32_t)(first - a0) : 0u,
+                                                             mine ? n_k : 0u, k, p.s, feat);
+                    if (mine) cnt = c;
+                    again = 0;
+                }
                 while (again) {  // exact selection by the whole warp
                     const uint32_t l = __ffs(again) - 1;
                     again &= again - 1;
@@ -416,7 +427,12 @@ cudaError_t launch_sketch(const SketchParams& p, uint32_t n_seq, const uint8_t* 
     if (n_windows == 0) return cudaSuccess;
     const int r = sketch_r_for(p.w);
     const char* name = EMIT ? "sketch_emit" : "sketch";
-    if (p.s <= LS_MAX_S) {
+    // Where a window's smallest hashes mostly repeat, as of 4^k / 2 canonical
+    // k-mers a window of n holds s n / (4^k / 2) repeats of one of its s
+    // smallest, most windows need the exact selection, and the kernel that
+    // makes no other is faster (k = 4, 64 Mbp: 339 us, 410 with lanes).
+    const bool repeats = 4ull * p.s * (p.w - p.k + 1) > 1ull << (2 * p.k);
+    if (p.s <= LS_MAX_S && !repeats) {
         using Kernel = void (*)(SketchParams, uint32_t, const uint8_t*, const uint64_t*, const uint64_t*, uint64_t,
                                 uint32_t, uint32_t, uint64_t*, uint32_t*, uint32_t*, unsigned long long*);
         const bool k16 = p.k == 16;

@@ -539,6 +539,87 @@ __device__ __forceinline__ bool lane_sketch(const uint32_t* code, const uint16_t
     return !over && !dup && (C >= p.s || tau == 0xFFFFFFFFu);
 }
 
+// The exact selection with one window per lane, for the windows that
+// lane_sketch leaves (n_k = 0: not this lane's; all lanes call together): a
+// lane keeps its 16 smallest distinct hashes sorted in registers.  A k-mer
+// that is new to no lane costs the hash, 16 compares and a vote, one that is
+// another 32 minimum and maximum steps.  Writes the features to the lane's
+// column of feat (stride LS_FEAT_STRIDE) and returns their number.
+// Sequence without variety leaves most windows of a warp, and the exact
+// selection by the whole warp takes them one by one: 64 Mbp of a repeat of six
+// bases 527 us that
+// way, 271 this way, of N 336 and 107.
+template <int KC>
+__device__ __forceinline__ uint32_t lane_sketch_exact(const uint32_t* code, const uint16_t* inv, uint32_t n_words,
+                                                   uint32_t pos, uint32_t n_k, uint32_t k_any, uint32_t s,
+                                                   uint32_t* feat) {
+    const uint32_t lane = lane_id();
+    const uint32_t k = KC ? (uint32_t)KC : k_any;
+    const uint32_t n_max = __reduce_max_sync(FULL_MASK, n_k);
+    const uint32_t last = n_words - 1;
+    const uint32_t boff = pos & 15u, sh = 2 * boff;
+    uint32_t wi = pos >> 4;
+    uint32_t w1 = code[min(wi + 1, last)];
+    uint32_t a0 = __funnelshift_l(w1, code[min(wi, last)], sh);
+    uint32_t r0 = revcomp16(a0);
+    uint32_t v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0xFFFFFFFFu;
+    bool ones = false;  // the hash of all ones, which marks a free place too, was met
+    for (uint32_t base = 0; base < n_max; base += 16, ++wi) {
+        const uint32_t w2 = code[min(wi + 2, last)];
+        const uint32_t a1 = __funnelshift_l(w2, w1, sh);
+        const uint32_t r1 = revcomp16(a1);
+        // bit 15 - r: k-mer base + r exists and holds no invalid base
+        const uint32_t rem = n_k > base ? n_k - base : 0u;
+        uint32_t ok = rem >= 16 ? 0xFFFFu : (0xFFFF0000u >> rem) & 0xFFFFu;
+        const uint32_t hi = ((uint32_t)inv[min(wi, last)] << 16) | inv[min(wi + 1, last)];
+        uint32_t z = __funnelshift_l((uint32_t)inv[min(wi + 2, last)] << 16, hi, boff);
+        uint32_t c = 1;
+        for (; 2 * c <= k; c *= 2) z |= z << c;
+        z |= z << (k - c);
+        ok &= ~(z >> 16);
+        if (__any_sync(FULL_MASK, ok != 0)) {
+#pragma unroll 1
+            for (uint32_t r = 0; r < 16; ++r) {
+                uint32_t f = __funnelshift_l(a1, a0, 2 * r);
+                uint32_t g = __funnelshift_r(r0, r1, 2 * r);
+                if (KC == 0) {
+                    f >>= 32 - 2 * k;
+                    g &= 0xFFFFFFFFu >> (32 - 2 * k);
+                }
+                uint32_t y = hash_h1(min(f, g));
+                bool in = (ok >> (15 - r)) & 1u;
+                ones |= in && y == 0xFFFFFFFFu;
+                in = in && y < v[15];
+#pragma unroll
+                for (int i = 0; i < 15; ++i) in = in && y != v[i];
+                if (__any_sync(FULL_MASK, in)) {
+                    if (!in) y = 0xFFFFFFFFu;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const uint32_t x = v[i];
+                        v[i] = min(x, y);
+                        y = max(x, y);
+                    }
+                }
+            }
+        }
+        a0 = a1;
+        r0 = r1;
+        w1 = w2;
+    }
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) cnt += (uint32_t)i < s && v[i] != 0xFFFFFFFFu;
+    cnt = min(cnt + (ones ? 1u : 0u), s);
+    if (n_k) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) feat[i * LS_FEAT_STRIDE + lane] = v[i];
+    }
+    return cnt;
+}
+
 // R for a window length: the warp covers 32*R >= w bases.
 __host__ __device__ inline int sketch_r_for(uint32_t w) { return w <= 128 ? 4 : (w <= 256 ? 8 : 16); }
 
