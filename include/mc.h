@@ -303,14 +303,18 @@ typedef struct mc_batch {
  *                locations as they are stored (32 or 64 bits); with
  *                wide_keys 1 on 32-bit locations the hash path is used.
  *  sort_max    : sort path: largest number of gathered locations a query
- *                may have to be sorted, 256, 512, 1024 (default) or 2048; each
- *                size class up to it has its own kernel; larger queries go
- *                to the hash path's medium and large kernels.
+ *                may have to be sorted, 256, 512, 1024 (default) or 2048 (with
+ *                64-bit locations the same as 1024); each size class up to it
+ *                has its own kernel; larger queries are queued.
  *  hist_slots  : hash path: shared-memory histogram slots per query: 256,
- *                512 (default) or 1024.  Queries whose distinct locations
- *                do not fit go to the medium (2,048 slots) and large paths.
- *  probe_batch : feature-table probes in flight per lane (32 lanes probe
- *                together): 2 (default), 4 or 8.
+ *                512 (default) or 1024.  Queries with more locations, or whose
+ *                distinct locations do not fit, are queued.
+ *                Queued queries of up to 1,024 locations are sorted by a warp
+ *                each (where sort_max or hist_slots is below that), the rest
+ *                take the medium path: a CTA each, up to 1,536 distinct
+ *                locations that can matter, and beyond that the large path.
+ *  probe_batch : feature-table probes in flight per lane: 2 (default), 4 or
+ *                8.
  *  gather_batch: hash path: bucket-location loads in flight per lane: 4, 8
  *                (default) or 16.
  *  lookup_warps: warps per CTA of the lookup kernel: 4 or 8 (default).
@@ -319,8 +323,10 @@ typedef struct mc_batch {
  *                by 32 bits (target << b | window) when every target and
  *                window id of the database fits 32 bits, else by 64; 1 =
  *                always 64-bit keys (hash path).
- * One warp carries one query on the sort and hash paths, one CTA beyond them
- * and in launches of at most 512 queries, which ignore the shape. */
+ * One warp carries one query on the sort and hash paths, one CTA beyond them.
+ * Launches of few queries ignore the shape and give every query a CTA: up to
+ * 512 queries, or 304 with 64-bit locations (mc_classify_noalloc: 16 and 8),
+ * in one call or one run of a plan, without counters. */
 typedef struct mc_tuning {
     uint32_t hist_slots;
     uint32_t probe_batch;
@@ -347,8 +353,8 @@ int mc_classify_batches(const mc_db* db, const mc_classify_params* params, const
 
 /* A reusable classification plan: scratch memory for up to max_queries
  * queries in up to max_batches batches, and a CUDA graph of the whole
- * launch set, captured once (for runs of few queries beside the plan's
- * capacity, graphs of their own, captured with the first such run).
+ * launch set, captured once (and graphs of their own for runs of fewer
+ * queries than it holds).
  * mc_plan_run replays the graph for a new set
  * of batches: it copies the batch descriptors (host, n_batches) to the
  * device and launches the graph on `stream`.  A plan is re-captured
@@ -369,6 +375,8 @@ void mc_plan_free(mc_plan* plan);
  * sort_max, each with the medium and large paths it leaves) on the given
  * sample batches (at most 2^20 queries
  * in total), `reps` times each, and writes the fastest setting to *best.
+ * The kernels depend on the number of queries (up to 512, below 16,384, and
+ * more), so a sample tells about launches in its own range.
  * If `times` is not NULL it receives up to max_times records
  * {setting, kernel ms (mean over reps)} in the order tried; *n_times (if
  * not NULL) the number tried.  Synchronises the database stream. */
@@ -478,7 +486,8 @@ void mc_server_free(mc_server* srv);
 /* Synchronises `stream` and returns (and clears) the first device-detected
  * error of earlier mc_classify calls of this database (MC_ERR_CAPACITY for
  * a query with more distinct hit locations than the largest per-query
- * histogram holds, or more windows than MC_MAX_QUERY_WINDOWS). */
+ * histogram holds, of which more than 2,048 could matter to its label (or
+ * candidate list), or with more windows than MC_MAX_QUERY_WINDOWS). */
 int mc_classify_status(const mc_db* db, void* stream);
 
 /* Releases the database and all its device memory (synchronises its stream). */
@@ -560,11 +569,13 @@ int mc_sketch(const mc_db_params* params, uint32_t n_seq, const char* seq, const
  * [0] features looked up, [1] locations gathered, [2] distinct locations,
  * [3] queries sent to the large-histogram path, [4] features found, [5]
  * 32-byte sectors of the gathered buckets, [6] queries finished on the
- * medium-histogram path; then per scoring kernel k (0 hash-path score
+ * medium path; then per scoring kernel k (0 hash-path score
  * kernel, 1-3 sort path for up to 256/512/1024 locations, 4 medium path,
  * 5 large path, 6 sort path for up to 2048 locations): [7 + 3k] queries it
  * finished, [8 + 3k] their found features, [9 + 3k] their 32-byte
- * sectors. */
+ * sectors.  So that all distinct locations are counted, a call with counters
+ * drops none before the sort, takes the hash path with 64-bit locations, and
+ * launches few queries as it does many. */
 #define MC_DEBUG_COUNTERS 28
 int mc_classify_debug(const mc_db* db, const mc_classify_params* params, uint32_t n_seq, const char* seq,
                       const uint64_t* offs, uint32_t n_queries, const uint32_t* qoffs, uint32_t* label,

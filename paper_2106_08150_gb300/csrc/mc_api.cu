@@ -1176,8 +1176,8 @@ struct mc_plan {
     unsigned char* host = nullptr;  // pinned image of the descriptors
     cudaStream_t cap = nullptr;     // capture stream
     // The launch set for at most n_q queries.  A run takes the smallest that
-    // holds its queries; the largest is captured with the plan, the others on
-    // their first use.
+    // holds its queries.  All are captured with the plan (no run waits for
+    // one) and again with their first use after the database changed.
     struct Set {
         uint32_t n_q = 0;
         cudaGraph_t graph = nullptr;
@@ -1320,8 +1320,10 @@ int mc_plan_create(const mc_db* db, const mc_classify_params* params, const mc_t
     if ((e = cudaStreamSynchronize(db->stream)) != cudaSuccess) return bail(cuda_fail(e, "mc_plan_create"));
     uint32_t sizes[mc::CLASSIFY_MAX_SIZES];
     p->n_sets = mc::classify_set_sizes(db_view(db), p->sc, sizes);
-    for (int i = 0; i < p->n_sets; ++i) p->sets[i].n_q = sizes[i];
-    if ((rc = plan_capture(p, p->sets[p->n_sets - 1]))) return bail(rc);
+    for (int i = 0; i < p->n_sets; ++i) {
+        p->sets[i].n_q = sizes[i];
+        if ((rc = plan_capture(p, p->sets[i]))) return bail(rc);
+    }
     *out = p;
     return MC_OK;
 }
