@@ -444,7 +444,7 @@ cudaError_t launch_sketch(const SketchParams& p, uint32_t n_seq, const uint8_t* 
         if (e != cudaSuccess) return e;
         // rounds of 32 windows per task: 16 where there are windows enough
         // for every resident warp, fewer in small calls
-        const uint64_t warps = (uint64_t)NUM_SMS_HINT * 5 * EMIT_WARPS;
+        const uint64_t warps = (uint64_t)NUM_SMS_HINT * EMIT_CTAS * EMIT_WARPS;
         const uint64_t rounds = (n_windows + 32 * warps - 1) / (32 * warps);
         const uint32_t task_windows = 32u * (uint32_t)(rounds < 16 ? rounds : 16);
         const uint64_t tasks = (n_windows + task_windows - 1) / task_windows;

@@ -33,7 +33,7 @@ namespace {
 constexpr int CLS_WARPS = 4;                 // warps per CTA (score path)
 constexpr int LK_WARPS = 8;                  // warps per CTA (lookup path)
 constexpr int WIN_A = 8;                     // windows per query on the shared-memory path
-constexpr uint32_t KB_SLOTS = 1u << 16;      // large-path histogram slots per warp
+constexpr uint32_t KB_SLOTS = 1u << 16;      // large-path histogram slots per CTA
 constexpr uint32_t LIST_B = MC_MAX_QUERY_WINDOWS * MAX_S;
 constexpr uint32_t LIST_CAP_MAX = WIN_A * MAX_S;  // bucket list of a query of the lookup kernels, any sketch size
 constexpr uint32_t MED_DISTINCT = 1536;      // distinct locations of a query on the medium path
@@ -2649,7 +2649,7 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
                 compact ? SortMem<64, uint32_t>::bytes(lc) : 0};
             return SORT_WARPS * b[c2];
         };
-        const uint32_t largest = compact ? t.sort_max : std::min(t.sort_max, 1024u);  // 64-bit keys: registers
+        const uint32_t largest = compact ? t.sort_max : std::min(t.sort_max, 1024u);  // 64-bit: registers
         // groups of 32 queries where every resident warp gets several,
         // smaller ones in small launches, down to one query per warp
         const uint64_t warps = (uint64_t)sms * 28;
@@ -3171,9 +3171,11 @@ cudaError_t classify_autotune(const ClassifyDb& db, const ClassifyQuery& Q, cons
                 }
             }
         }
-        // the sort path, for each largest size class
+        // the sort path, for each largest size class (64-bit locations have
+        // no larger one than 1,024: 2,048 would be timed twice)
         {
             for (uint32_t smax : {256u, 512u, 1024u, 2048u}) {
+                if (smax > 1024 && !db.jbits) break;
                 Tuning t = cur;
                 t.score_mode = SCORE_SORT;
                 t.sort_max = smax;

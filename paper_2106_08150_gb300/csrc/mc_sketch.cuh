@@ -547,8 +547,7 @@ __device__ __forceinline__ bool lane_sketch(const uint32_t* code, const uint16_t
 // column of feat (stride LS_FEAT_STRIDE) and returns their number.
 // Sequence without variety leaves most windows of a warp, and the exact
 // selection by the whole warp takes them one by one: 64 Mbp of a repeat of six
-// bases 527 us that
-// way, 271 this way, of N 336 and 107.
+// bases 527 us that way, 271 this way, of N 336 and 107.
 template <int KC>
 __device__ __forceinline__ uint32_t lane_sketch_exact(const uint32_t* code, const uint16_t* inv, uint32_t n_words,
                                                    uint32_t pos, uint32_t n_k, uint32_t k_any, uint32_t s,

@@ -94,3 +94,20 @@ def test_counting_call(mc, wide):
     assert [int(ctr[i]) for i in range(3)] == [int(want[3][:, i].sum()) for i in range(3)]
     bases = np.array([sum(map(len, q)) for q in qs])
     assert int(ctr[7]) >= int(((want[3][:, 1] <= 256) & (bases <= 900)).sum()) > 200  # it holds 384 distinct
+
+
+def test_autotuner_times_each_shape_once(mc, wide):
+    """64-bit locations have no size class beyond 1,024."""
+    import torch
+    db, odb, parent, taxon, qs = wide
+    reads, roffs, qoffs = sf._reads(qs)
+    out = [torch.zeros(len(qs), dtype=torch.int32, device="cuda") for _ in range(3)]
+    b = mc.batch(len(roffs) - 1, dev(reads), dev(roffs), dev(qoffs), *out)
+    cp = mc.classify_params(**CLS)
+    best, rec = mc.mc_autotune(db.handle, cp, [b], reps=1)
+    assert len(rec) == 6 + 18 + 3
+    mc.mc_classify_batches(db.handle, cp, [b], best)
+    mc.mc_classify_status(db.handle)
+    want = odb.classify(parent, taxon, reads, roffs, qoffs, max_candidates=4, n_threads=8, **CLS)
+    for g, o in zip(out, want):
+        assert (host_u32(g) == o).all()
