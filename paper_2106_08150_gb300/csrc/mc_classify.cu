@@ -719,6 +719,22 @@ __device__ __forceinline__ void flush_counters(const ClassifyQuery& Q, const Cou
     }
 }
 
+// The counters of a warp's queries in a counting call (COUNTING kernels), kept
+// in shared memory by its lane 0 and added up once: added per query, on eight
+// addresses, they took longer than the sort (10^6 pairs, smallest class: 5.4
+// ms that way, 1.6 this way).
+__device__ __forceinline__ void flush_tally(const ClassifyQuery& Q, const unsigned long long* tally, int kidx) {
+    if (lane_id()) return;
+    Counters c;
+    c.features = tally[0];
+    c.locations = tally[1];
+    c.distinct = tally[2];
+    c.found = tally[3];
+    c.sectors = tally[4];
+    c.queries = tally[5];
+    flush_counters(Q, c, kidx);
+}
+
 constexpr uint32_t BUF_A = 1024;   // bases per query on the shared-memory path
 constexpr uint32_t BUF_B = 16384;  // bases per query on the large path
 
@@ -803,6 +819,17 @@ __device__ __forceinline__ void note_widest(uint32_t* widest, uint32_t locations
 constexpr uint32_t META_FEAT_SHIFT = 20;
 __device__ __forceinline__ uint32_t meta_sws(const uint4& m) { return m.y & ((1u << META_FEAT_SHIFT) - 1u); }
 __device__ __forceinline__ uint32_t meta_feat(const uint4& m) { return m.y >> META_FEAT_SHIFT; }
+
+__device__ __forceinline__ void tally_query(unsigned long long* tally, const uint4& mt, uint32_t distinct) {
+    __syncwarp();
+    if (lane_id()) return;
+    tally[0] += meta_feat(mt);
+    tally[1] += mt.z;
+    tally[2] += distinct;
+    tally[3] += mt.x;
+    tally[4] += mt.w;
+    tally[5] += 1;
+}
 
 // Main path, part 1 (sketch + lookup): one warp per query of the chunk
 // [q0, q0 + nq), shared memory for the query's bases and features only, so
@@ -1748,7 +1775,7 @@ __device__ __forceinline__ uint32_t score_sorted(const ClassifyDb& db, const Cla
 // locations (64-bit locations): the query goes to the medium path.
 template <int E, class LocT>
 __device__ __forceinline__ bool query_sort(const ClassifyDb& db, const ClassifyQuery& Q, uint32_t q,
-                                          const SortMem<E, LocT>& M, uint32_t sws, uint32_t H,
+                                          const SortMem<E, LocT>& M, uint32_t sws, uint32_t H, bool counting,
                                           uint32_t& distinct) {
     using Mem = SortMem<E, LocT>;
     constexpr uint32_t MASK = Mem::CAP - 1;  // block counters
@@ -1762,7 +1789,7 @@ __device__ __forceinline__ bool query_sort(const ClassifyDb& db, const ClassifyQ
     LocT* const raw = M.raw;
     LocT* surv = reinterpret_cast<LocT*>(M.b);
     // the counters of mc_classify_debug count all distinct locations
-    uint32_t T = (H <= NO_FILTER || Q.counters) ? 1u : 0u;
+    uint32_t T = (H <= NO_FILTER || counting) ? 1u : 0u;
     do {
         const LocT* from = raw;
         uint32_t n = H;
@@ -1916,7 +1943,7 @@ constexpr int sort_min_ctas() {
 // Sort path over the chunk's queries with h_lo < H <= 32*E gathered
 // locations; with last (the largest class), larger ones are queued for the
 // medium path.
-template <int E, class LocT>
+template <int E, class LocT, bool COUNTING>
 __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     k_classify_sort(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t chunk, uint32_t list_cap,
                     const uint64_t* __restrict__ glist, const uint4* __restrict__ meta, uint32_t h_lo, bool last,
@@ -1925,6 +1952,8 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t w = threadIdx.x >> 5;
     const SortMem<E, LocT> M(smem + w * SortMem<E, LocT>::bytes(list_cap), list_cap);
+    __shared__ unsigned long long tally[COUNTING ? SORT_WARPS : 1][6];
+    if (COUNTING && lane_id() < 6) tally[w][lane_id()] = 0;
     // the next size class, which shares no data with this one, may start
     // while this one's last queries finish
     asm volatile("griddepcontrol.launch_dependents;");
@@ -1943,21 +1972,15 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
                 sort_gather<E>(db, M, src, mt.x, mt.z);
                 cp_async_wait_all();
                 __syncwarp();
-                done = query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct);
+                done = query_sort<E>(db, Q, q0 + i, M, meta_sws(mt), mt.z, COUNTING, distinct);
             }
             if (!done) {
                 if (lane_id() == 0) mid_list[atomicAdd(mid_n, 1u)] = i;
-            } else if (Q.counters) {  // per query: a debug call need not keep them in registers
-                Counters ctr;
-                ctr.features = meta_feat(mt);
-                ctr.locations = mt.z;
-                ctr.distinct = distinct;
-                ctr.found = mt.x;
-                ctr.sectors = mt.w;
-                ctr.queries = 1;
-                flush_counters(Q, ctr, E == 8 ? 1 : (E == 16 ? 2 : (E == 32 ? 3 : 6)));
+            } else if (COUNTING) {
+                tally_query(tally[w], mt, distinct);
             }
         }
+        if (COUNTING) flush_tally(Q, tally[w], E == 8 ? 1 : (E == 16 ? 2 : (E == 32 ? 3 : 6)));
     }
     // Launched as a programmatic dependent of the medium path or of another
     // size class, this kernel may run alongside it; waiting for that grid
@@ -1974,15 +1997,17 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<E, LocT>())
 // each is slow (200,000 mixed reads, 1,000 genomes, sort_max 256: 4.66 ms, here
 // 0.98; score_mode 2 with 256 slots: 4.87 ms, here 1.22).  Lines of 1,024 leave
 // few that a warp could take, and the kernel is not launched.
-template <class LocT>
+template <class LocT, bool COUNTING>
 __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<32, LocT>())
     k_sort_queued(ClassifyDb db, ClassifyQuery Q, uint32_t q0, uint32_t list_cap, const uint64_t* __restrict__ glist,
                   const uint4* __restrict__ meta, const uint32_t* __restrict__ mid_list,
                   const uint32_t* __restrict__ mid_n, uint32_t* __restrict__ work, uint32_t* __restrict__ rest_list,
                   uint32_t* __restrict__ rest_n) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t lane = lane_id();
-    const SortMem<32, LocT> M(smem + (threadIdx.x >> 5) * SortMem<32, LocT>::bytes(list_cap), list_cap);
+    const uint32_t lane = lane_id(), w = threadIdx.x >> 5;
+    const SortMem<32, LocT> M(smem + w * SortMem<32, LocT>::bytes(list_cap), list_cap);
+    __shared__ unsigned long long tally[COUNTING ? SORT_WARPS : 1][6];
+    if (COUNTING && lane < 6) tally[w][lane] = 0;
     const uint32_t n = *mid_n;
     for (;;) {
         uint32_t k = 0;
@@ -1997,21 +2022,17 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<32, LocT>())
             sort_gather<32>(db, M, glist + (uint64_t)i * list_cap, mt.x, mt.z);
             cp_async_wait_all();
             __syncwarp();
-            done = query_sort<32>(db, Q, q0 + i, M, meta_sws(mt), mt.z, distinct);
+            done = query_sort<32>(db, Q, q0 + i, M, meta_sws(mt), mt.z, COUNTING, distinct);
         }
         if (!done) {
             if (lane == 0) rest_list[atomicAdd(rest_n, 1u)] = i;
-        } else if (Q.counters) {
-            Counters ctr;
-            ctr.features = meta_feat(mt);
-            ctr.locations = mt.z;
-            ctr.distinct = distinct;
-            ctr.found = mt.x;
-            ctr.sectors = mt.w;
-            ctr.queries = 1;
-            flush_counters(Q, ctr, KC_MEDIUM);
-            if (lane == 0) atomicAdd(Q.counters + 6, 1ull);
+        } else if (COUNTING) {
+            tally_query(tally[w], mt, distinct);
         }
+    }
+    if (COUNTING) {
+        flush_tally(Q, tally[w], KC_MEDIUM);
+        if (lane == 0) atomicAdd(Q.counters + 6, tally[w][5]);
     }
 }
 
@@ -2218,7 +2239,8 @@ __device__ __forceinline__ bool block_score(const ClassifyDb& db, const Classify
 }
 
 // Medium path: the queries queued by the hash path's score kernel or the
-// sort path's classes, one CTA each (work queue), the bucket list taken
+// sort path's classes, less those that k_sort_queued took; one CTA each (work
+// queue), the bucket list taken
 // over from the lookup; queries of more than MED_DISTINCT distinct locations
 // go to the large path.
 template <class LocT>
@@ -2637,10 +2659,14 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
     g->group_shift = 0;
     if (g->sort) {
         const SortKernel kts[N_SORT_CLASSES] = {
-            compact ? k_classify_sort<8, uint32_t> : k_classify_sort<8, uint64_t>,
-            compact ? k_classify_sort<16, uint32_t> : k_classify_sort<16, uint64_t>,
-            compact ? k_classify_sort<32, uint32_t> : k_classify_sort<32, uint64_t>,
-            compact ? k_classify_sort<64, uint32_t> : nullptr};
+            !compact ? k_classify_sort<8, uint64_t, false>
+                     : (counting ? k_classify_sort<8, uint32_t, true> : k_classify_sort<8, uint32_t, false>),
+            !compact ? k_classify_sort<16, uint64_t, false>
+                     : (counting ? k_classify_sort<16, uint32_t, true> : k_classify_sort<16, uint32_t, false>),
+            !compact ? k_classify_sort<32, uint64_t, false>
+                     : (counting ? k_classify_sort<32, uint32_t, true> : k_classify_sort<32, uint32_t, false>),
+            !compact ? nullptr
+                     : (counting ? k_classify_sort<64, uint32_t, true> : k_classify_sort<64, uint32_t, false>)};
         const auto bytes = [&](int c2, uint32_t lc) {
             const size_t b[N_SORT_CLASSES] = {
                 compact ? SortMem<8, uint32_t>::bytes(lc) : SortMem<8, uint64_t>::bytes(lc),
@@ -2676,7 +2702,8 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
         const auto bytes = [&](uint32_t lc) {
             return SORT_WARPS * (db.jbits ? SortMem<32, uint32_t>::bytes(lc) : SortMem<32, uint64_t>::bytes(lc));
         };
-        g->kq = db.jbits ? k_sort_queued<uint32_t> : k_sort_queued<uint64_t>;
+        g->kq = db.jbits ? (counting ? k_sort_queued<uint32_t, true> : k_sort_queued<uint32_t, false>)
+                         : (counting ? k_sort_queued<uint64_t, true> : k_sort_queued<uint64_t, false>);
         g->smem_q = bytes(g->list_cap);
         if ((e = allow_smem(g->kq, bytes(LIST_CAP_MAX))) != cudaSuccess) return e;
         int occ_q = 1;
@@ -2749,9 +2776,11 @@ cudaError_t launch_medium(const Geometry& g, const ClassifyDb& db, const Classif
 
 // A launch of few queries: all of them straight to the large path's kernel.
 // One launch instead of the six kernels and a memset of a launch set,
-// whose latency is what such a call takes: 16 pairs 25 us on the device
-// against 65.  One wave of CTAs (two per SM) holds 304 queries; 2,000 take
-// 115 us this way and 61 the other (reads of 100), so the line lies between.
+// whose latency is what such a call takes: 16 pairs 23 us on the device
+// against some 40.  One wave of CTAs (two per SM) holds 304 queries; a second
+// is faster or slower than the launch set by the reads (512 queries this way,
+// 600 the other: mixed reads, related genomes 46 and 55 us, repeat-rich genomes
+// 99 and 113, reads of 100 40 and 35), and the line lies within it.
 // With 64-bit locations a launch set is shorter (one size class), and the line
 // is one wave: pairs of 100, draft assemblies, 200 queries 23 us this way and
 // 30 the other, 400 queries 38 and 31 (54 and 37 with candidate lists).
