@@ -2057,30 +2057,50 @@ constexpr uint32_t BLK_DISTINCT = 2048;                      // of which as many
 constexpr int BLK_CTAS = 2;                                  // resident per SM
 constexpr int BLK_STEP = 8;                                  // consecutive locations per thread and step
 
+// The block counters and the sorted distinct survivors.  With 64-bit locations
+// the survivors take the counters' place, without which two CTAs do not fit
+// an SM (a query that is done again then counts again: 2 to 6 us).
 template <class LocT>
-struct BlockMem {
+struct BlockCounters {
+    uint32_t cnt[BLK_CNT];
+    LocT loc[BLK_DISTINCT];
+};
+template <>
+struct BlockCounters<uint64_t> {
+    union {
+        uint32_t cnt[BLK_CNT];
+        uint64_t loc[BLK_DISTINCT];
+    };
+};
+
+template <class LocT>
+struct BlockMem : BlockCounters<LocT> {
     uint64_t list[BLK_LIST];      // found buckets, offset << 16 | size
     uint32_t pre[BLK_LIST + 4];   // exclusive prefix of their sizes
     union {
-        uint32_t cnt[BLK_CNT];    // block counters, until the survivors are chosen
-        LocT loc[BLK_DISTINCT];   // the distinct survivors, sorted
+        LocT key[BLK_HASH];       // the distinct survivors, hashed (times: how often each was gathered)
+        struct {                  // (before them) the lookup's windows:
+            uint64_t waddr[MC_MAX_QUERY_WINDOWS];  // address of the first base,
+            uint32_t wnk[MC_MAX_QUERY_WINDOWS];    // k-mers, features
+            uint32_t wcnt[MC_MAX_QUERY_WINDOWS];
+            uint32_t cand[BLK_WARPS][32];
+        };
     };
-    LocT key[BLK_HASH];           // the distinct survivors, hashed,
-    uint32_t times[BLK_HASH];     // and how often each was gathered
+    uint32_t times[BLK_HASH];
     uint32_t rs[BLK_DISTINCT + 4];
     union {
         uint32_t score[BLK_DISTINCT + 4];
         uint32_t feat[BLK_LIST];  // (before the scores) the windows' features
     };
-    uint64_t waddr[MC_MAX_QUERY_WINDOWS];  // windows: address of the first base,
-    uint32_t wnk[MC_MAX_QUERY_WINDOWS];    // k-mers, features
-    uint32_t wcnt[MC_MAX_QUERY_WINDOWS];
-    uint32_t cand[BLK_WARPS][32];
     uint32_t part[BLK_WARPS];     // block-wide scan and maximum
     uint32_t n_list, sect, n, T, n_win, sws, n_feat, work;
     int status;
 };
 
+// Two CTAs within 196 KB, the largest shared memory of an SM but one, leave it
+// 60 KB of L1 instead of 28 (5,000 reads of 1 to 6 kbp: 0.72 ms instead of
+// 0.87).
+static_assert(BLK_CTAS * (sizeof(BlockMem<uint32_t>) + 1024) <= 196 * 1024, "shared memory of an SM");
 static_assert(BLK_CTAS * (sizeof(BlockMem<uint64_t>) + 1024) <= 228 * 1024, "shared memory of an SM");
 
 // f(location) for every location of the query's n_list buckets (H in all).
@@ -2234,7 +2254,7 @@ __device__ __forceinline__ bool block_score(const ClassifyDb& db, const Classify
         T = B.T;
         distinct = D;
         if (T == 0) return true;
-        if (T > 1) block_count_again<LocT>(db, B, n_list, H, bs);  // (the survivors took the counters' place)
+        if (sizeof(LocT) == 8 && T > 1) block_count_again<LocT>(db, B, n_list, H, bs);
     }
 }
 
