@@ -2047,7 +2047,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32, sort_min_ctas<32, LocT>())
 // One warp per query with a histogram took 0.6 ms for the slowest of a
 // launch of 2^20 pairs, whatever the others did (large database, 2 launches
 // 1.24 ms, here 0.71), and 5,000 reads of 1 to 6 kbp took 9.05 ms on
-// global-memory histograms, here 0.82.
+// global-memory histograms, here 0.72.
 constexpr int BLK_THREADS = 256;
 constexpr int BLK_WARPS = BLK_THREADS / 32;
 constexpr uint32_t BLK_LIST = MC_MAX_QUERY_WINDOWS * MAX_S;  // buckets of one query
@@ -2736,7 +2736,8 @@ cudaError_t geometry(const ClassifyDb& db, const Tuning& t, const ClassifyScratc
 __host__ __device__ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scratch layout: escalation queue + counters, chunk metadata, medium-path
-// queue and the queue of what warps leave of it, chunk bucket lists, large-path working memory.
+// queue and the queue of what warps leave of it, chunk bucket lists,
+// large-path working memory.
 struct ScratchLayout {
     size_t ovf, meta, mid, glist, large, total;
     uint32_t chunk;
@@ -2829,8 +2830,9 @@ cudaError_t reset_counters(const ClassifyScratch& sc, int from, int to, cudaStre
     return cudaMemsetAsync(queue_counters(sc) + from, 0, (to - from) * sizeof(uint32_t), s);
 }
 
-// Score of the chunk at q0, whose counters QC_MID .. QC_WIDEST are zero (each
-// launch appends up to a chunk's queries to the queues).  Sort path, 32-bit locations: the largest size
+// Score of the chunk at q0, whose counters from QC_MID up to QC_WIDEST are zero
+// (each launch appends up to a chunk's queries to the queues).  Sort path,
+// 32-bit locations: the largest size
 // class first (it queues the queries beyond it), then the medium path, then
 // the other classes, the most populous one (512) first.  Each of those is
 // launched with programmatic stream serialization, so that it fills the SMs
